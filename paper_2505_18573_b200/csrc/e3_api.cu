@@ -3,6 +3,7 @@
 #include <stdint.h>
 
 #include "e3.h"
+#include "e3_internal.h"
 #include "e3_rows.cuh"
 #include "e3_small.cuh"
 
@@ -159,16 +160,28 @@ extern "C" e3_status e3_sequence_mean_entropy(const float *ent, const uint8_t *m
   return e == cudaSuccess ? E3_OK : E3_ERR_CUDA;
 }
 
-extern "C" e3_status e3_group_advantage(const float *rewards, const int64_t *group_offsets, int64_t n_groups,
-                                        float eps, int unbiased, float *out_adv, uint8_t *out_group_flags,
-                                        void *stream) {
+namespace {
+// n_fill >= 0: see e3::group_advantage_filled
+e3_status group_advantage(const float *rewards, const int64_t *group_offsets, int64_t n_groups, float eps, int unbiased,
+                          float *out_adv, uint8_t *out_group_flags, int64_t n_fill, void *stream) {
   if (n_groups < 0 || !(eps >= 0.f) || !(eps < 3.0e38f)) return E3_ERR_INVALID_ARG;
-  if (n_groups == 0) return E3_OK;
+  if (n_groups == 0 && n_fill <= 0) return E3_OK;
   if (!rewards || !group_offsets || !out_adv) return E3_ERR_INVALID_ARG;
   if (misaligned(rewards, 4) || misaligned(group_offsets, 8) || misaligned(out_adv, 4)) return E3_ERR_ALIGNMENT;
   cudaError_t e = e3::launch_group_advantage(rewards, group_offsets, n_groups, eps, unbiased, out_adv,
-                                             out_group_flags, static_cast<cudaStream_t>(stream));
+                                             out_group_flags, n_fill, static_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? E3_OK : E3_ERR_CUDA;
+}
+}  // namespace
+
+extern "C" e3_status e3_group_advantage(const float *rewards, const int64_t *group_offsets, int64_t n_groups,
+                                        float eps, int unbiased, float *out_adv, uint8_t *out_group_flags,
+                                        void *stream) {
+  return group_advantage(rewards, group_offsets, n_groups, eps, unbiased, out_adv, out_group_flags, -1, stream);
+}
+e3_status e3::group_advantage_filled(const float *rewards, int64_t n_rewards, const int64_t *group_offsets, int64_t n_groups,
+                                     float eps, int unbiased, float *out_adv, uint8_t *out_group_flags, void *stream) {
+  return group_advantage(rewards, group_offsets, n_groups, eps, unbiased, out_adv, out_group_flags, n_rewards, stream);
 }
 
 extern "C" void e3_test_arm_stall(int64_t tile, uint64_t wait_ns) { e3::arm_stall(tile, wait_ns); }

@@ -23,11 +23,6 @@ e3_status check_logits(const void *logits, e3_dtype dt, int64_t rows, int64_t V,
   return E3_OK;
 }
 
-bool rows_are_16B_aligned(const void *logits, e3_dtype dt, int64_t row_stride) {
-  const int64_t esize = dt == E3_F32 ? 4 : 2;
-  return !misaligned(logits, 16) && (row_stride * esize) % 16 == 0;
-}
-
 void philox_round_keys(uint64_t seed, uint32_t rk[20]) {
   uint32_t k0 = static_cast<uint32_t>(seed), k1 = static_cast<uint32_t>(seed >> 32);
   for (int r = 0; r < 10; ++r) {
@@ -75,7 +70,7 @@ extern "C" e3_status e3_sample(const void *logits, e3_dtype dt, int64_t rows, in
     return E3_ERR_WORKSPACE;
 
   e3::RowsParams p = {};
-  p.logits = logits; p.rows = rows; p.V = V; p.row_stride = row_stride;
+  p.logits = static_cast<const char *>(logits); p.V = (int)V; p.row_bytes = row_stride * (dt == E3_F32 ? 4 : 2);
   p.temps = temps; p.temp_scalar = 1.f;
   p.out_tok = out_tok; p.out_logp = out_logp; p.out_ent = out_ent; p.out_gap = out_gap; p.status = out_status;
   philox_round_keys(seed, p.round_key);
@@ -84,9 +79,8 @@ extern "C" e3_status e3_sample(const void *logits, e3_dtype dt, int64_t rows, in
   p.row_base = static_cast<uint32_t>(row_base);
   p.mode = e3::kModeSample;
   p.slack_scale = sampler == E3_SAMPLER_TOKEN_AUDIT ? 1000.f : 1.f;
-  cudaError_t e = e3::launch_rows(p, static_cast<int>(dt), sampler == E3_SAMPLER_BLOCK ? 1 : 0,
-                                  rows_are_16B_aligned(logits, dt, row_stride), workspace, workspace_bytes,
-                                  static_cast<cudaStream_t>(stream));
+  cudaError_t e = e3::launch_rows(p, rows, static_cast<int>(dt), sampler == E3_SAMPLER_BLOCK ? 1 : 0, workspace,
+                                  workspace_bytes, static_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? E3_OK : E3_ERR_CUDA;
 }
 
@@ -117,15 +111,14 @@ extern "C" e3_status e3_token_logp_entropy(const void *logits, e3_dtype dt, int6
     return E3_ERR_ALIGNMENT;
 
   e3::RowsParams p = {};
-  p.logits = logits; p.rows = rows; p.V = V; p.row_stride = row_stride;
+  p.logits = static_cast<const char *>(logits); p.V = (int)V; p.row_bytes = row_stride * (dt == E3_F32 ? 4 : 2);
   p.temps = temps; p.temp_scalar = temp_scalar;
   p.targets = targets; p.mask = mask;
   p.out_logp = out_logp; p.out_ent = out_ent; p.out_gap = out_gap; p.status = out_status;
   p.mode = e3::kModeTargets;
   p.slack_scale = 1.f;
-  cudaError_t e = e3::launch_rows(p, static_cast<int>(dt), -1, rows_are_16B_aligned(logits, dt, row_stride),
-                                  workspace, workspace_bytes < token_mean_offset() ? workspace_bytes : token_mean_offset(),
-                                  cs);
+  cudaError_t e = e3::launch_rows(p, rows, static_cast<int>(dt), -1, workspace,
+                                  workspace_bytes < token_mean_offset() ? workspace_bytes : token_mean_offset(), cs);
   // The fused mean entropy: the two reduction kernels of e3_masked_mean_entropy behind the row kernel, chained by
   // programmatic dependent launch; the same blocks add the same values in the same order.
   if (e == cudaSuccess && fused_mean)

@@ -965,7 +965,9 @@ __global__ void __launch_bounds__(kThreads, 1) rows_kernel(const __grid_constant
               // Groups whose sum passed the gate: their entries above it, whatever the coarse byte.  While nothing is known
               // of the row's scores the gate is set just below the largest logit first, and again when those entries and the
               // ones with byte 255 have been scored.  Where many logits lie close to the largest (a high temperature, a flat
-              // row) the latter alone give as good a bound: scoring a tile's every entry cost as much as ten tiles' sums.
+              // row: three lanes of four have one in their first vector) the latter alone give as good a bound: scoring a
+              // tile's every entry cost as much as ten tiles' sums.
+              constexpr int kCrowd = 24;
               constexpr float kFirstGate = 0.00422f;  // e^-2 2^-5: two units of score below the sample's largest
               float gate_hi = CUDART_INF_F, first_thr = CUDART_INF_F;
 #pragma unroll 1
@@ -981,9 +983,12 @@ __global__ void __launch_bounds__(kThreads, 1) rows_kernel(const __grid_constant
                 uint32_t over = 0u;  // bit j: the lane's group j passes
 #pragma unroll
                 for (int j = 0; j < kG; ++j) over |= (Zg[j] > ethr ? 1u : 0u) << j;
-                if (look == 0 && __all_sync(kAll, over != 0u)) {
-                  over = 0u;
-                  gate = ethr = CUDART_INF_F;  // (none has been looked at)
+                if (look == 0) {
+                  const uint4 v[1] = {lds128(B)};
+                  if (__popc(__ballot_sync(kAll, vec_max<DT>(v) > gate)) > kCrowd) {
+                    over = 0u;
+                    gate = ethr = CUDART_INF_F;  // (none has been looked at)
+                  }
                 }
 #pragma unroll 1
                 while (__any_sync(kAll, over != 0u)) {  // one group per lane and round
@@ -1148,7 +1153,7 @@ constexpr int64_t kStripsPerCta = 4;
 // (4,096 rows: 12 tiles 537 us, 25 494).
 int strip_tiles(int64_t tiles_per_cta, int sampler) {
   const int64_t per_warp = tiles_per_cta / kWarps;
-  if (sampler == 0) return per_warp < 1 ? 1 : (int)(per_warp < 20 ? per_warp * 6 / 5 + 1 : 25);
+  if (sampler == 0) return per_warp < 1 ? 1 : (int)(per_warp < 23 ? per_warp + 2 : 25);
   if (per_warp < 2) return per_warp < 1 ? 1 : 2;
   return sampler < 0 && per_warp >= 32 ? 8 : 4;
 }
@@ -1166,8 +1171,9 @@ cudaError_t launch_one(RowsParams p, int64_t rows, void *workspace, size_t works
   p.spr = (int)spr;
   p.inv_spr = 1.0f / (float)spr;
   p.unit = can_cut ? 1 : (int)spr;
-  // the blocked sampler keeps the scores of 512 tiles' blocks (its strips are 1, 2 or 4 tiles long)
-  p.ring = SAMPLER == 1 && strip > 2 ? 2 * kRing / (int)strip : kRing;
+  // the blocked sampler keeps the scores of 512 tiles' blocks
+  p.ring = kRing;
+  while (SAMPLER == 1 && p.ring * strip > 512) p.ring /= 2;
   p.ws_pieces = can_cut ? static_cast<unsigned char *>(workspace) : nullptr;
   p.wait_ns = kDefaultWaitNs;
   const long long stall = g_stall_tile.exchange(-1);  // (row * tpr + tile within the row)

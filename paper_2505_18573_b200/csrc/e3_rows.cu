@@ -1144,18 +1144,20 @@ size_t pieces_bytes() { return (size_t)kMaxGrid * 2 * kPieceBytes; }
 // the SM's four schedulers.
 constexpr int64_t kStripsPerCta = 4;
 
-// Tiles per strip.  Taking a strip and handing in its record cost a warp about as many instructions as a tile's sums: longer
-// strips cost less, shorter ones spread better at the end of a run.  Measured with 151,936 bf16 entries a row, us for strips of
-// 1, 2 and 4 tiles: statistics 64 rows 17.1, 12.8, 13.8, 128 rows 20.1, 19.4, 16.3, 512 rows 39.4, 34.9, 33.9; sampler 1 64 rows
-// 21.4, 16.4, 18.0, 128 rows 25.6, 25.1, 21.6, 512 rows 58.8, 51.2, 46.8.  Sampler 0 pays about two tiles' time for every
-// stay of a warp with a row (a first bound of the scores, a last look at the queue): a strip a little longer than a warp's share of a
-// short run, so that one strip per warp is all (512 rows: strips of 6 tiles 95 us, 12 or 13 87, 15 94), 25 tiles in a long one
-// (4,096 rows: 12 tiles 537 us, 25 494).
-int strip_tiles(int64_t tiles_per_cta, int sampler) {
-  const int64_t per_warp = tiles_per_cta / kWarps;
-  if (sampler == 0) return per_warp < 1 ? 1 : (int)(per_warp < 23 ? per_warp + 2 : 25);
-  if (per_warp < 2) return per_warp < 1 ? 1 : 2;
-  return sampler < 0 && per_warp >= 32 ? 8 : 4;
+// Tiles per strip.  Strips of one length keep the warps of an SM in step, so that a run of a few strips per warp takes
+// whole waves: in a short run one strip per warp is all, the shortest that does it (151,936 bf16 entries a row, us for the lengths
+// below it, at it and behind it: statistics 256 rows 4 to 8 tiles 25.8, 26.8, 21.5, 21.9, 22.6, 512 rows 11 to 13 tiles 39.2,
+// 32.6, 33.6, 8 tiles 37.0; sampler 1 256 rows 35.2, 33.7, 27.5, 27.6, 28.5, 512 rows 45.9, 40.1, 40.2; sampler 0 512 rows 6, 12,
+// 13, 15 tiles 95, 87, 86, 94).  In a long run the waves dissolve: there a strip is as long as makes its own cost small (taking
+// it and handing in its record cost a warp about as many instructions as a tile's sums; for sampler 0 the first bound and the
+// last look at the queue cost twice that: 4,096 rows 12 tiles 537, 25 tiles 494), and for sampler 1 as short as the ring of block
+// scores asks for (4,096 rows 4, 6, 8 tiles 234, 266, 244; 1,024 rows 72, 75, 68).
+int strip_tiles(int64_t rows, int64_t tpr, int64_t ctas, int sampler) {
+  const int64_t per_warp = rows * tpr / ctas / kWarps, longest = sampler == 0 ? 25 : 13;
+  for (int64_t n = per_warp < 1 ? 1 : per_warp; n <= longest; ++n)
+    if (rows * ((tpr + n - 1) / n) <= ctas * kWarps) return (int)n;
+  if (sampler == 0) return 25;
+  return sampler == 1 && per_warp >= 32 ? 4 : 8;
 }
 
 template <int DT, int SAMPLER>
@@ -1164,7 +1166,7 @@ cudaError_t launch_one(RowsParams p, int64_t rows, void *workspace, size_t works
   cudaError_t e = resident_ctas<DT, SAMPLER>(ctas);
   if (e != cudaSuccess) return e;
   const int64_t tpr = ((int64_t)p.V + Fmt<DT>::kTileE - 1) / Fmt<DT>::kTileE;
-  const int64_t strip = strip_tiles(rows * tpr / ctas, SAMPLER), spr = (tpr + strip - 1) / strip;
+  const int64_t strip = strip_tiles(rows, tpr, ctas, SAMPLER), spr = (tpr + strip - 1) / strip;
   const bool can_cut = workspace != nullptr && workspace_bytes >= pieces_bytes();
   p.tpr = (int)tpr;
   p.strip_tiles = (int)strip;

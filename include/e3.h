@@ -186,8 +186,8 @@ E3_API e3_status e3_token_logp_entropy(const void *logits, e3_dtype dt, int64_t 
  *                 normaliser is taken from them: ln p_i = (z_i - z_tok)/tau + logp)
  *   g_logp, g_ent device float [rows]: upstream gradients; NULL = all zero
  *   dlogits       device, same element type as logits, row r starts at element r * dlogits_stride
- *                 (dlogits_stride >= V); must not overlap logits.  Rows and strides that are 16-byte
- *                 aligned on both sides take the vectorised path.
+ *                 (dlogits_stride >= V); must not overlap logits.  Rows whose logits and gradients
+ *                 lie equally far behind a 16-byte boundary take the vectorised path.
  * No workspace.  One pass: V entries read and V written per row.
  */
 E3_API e3_status e3_token_logp_entropy_backward(const void *logits, e3_dtype dt, int64_t rows, int64_t V,

@@ -114,3 +114,24 @@ def test_backward_training_chunk_at_full_width(e3):
     got = out[sub].float().cpu().numpy().astype(np.float64)
     assert np.all(np.abs(got - ref) <= 2e-3 * (np.abs(g_lp.cpu().numpy()[pick]) + 1)[:, None] + np.abs(ref) * 2.0 ** -8)
     assert torch.all(out[mask == 0] == 0)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("V, start", [(1, 1), (2, 3), (8191, 1), (8192, 3), (8195, 1), (8199, 1), (16385, 2), (16391, 7)])
+def test_backward_rows_off_a_16_byte_boundary(e3, dtype, V, start):
+    """Rows that begin anywhere behind a 16-byte boundary (the head, the vectors and the tail of every segment), with gradients
+    that lie equally far behind one and with gradients that do not."""
+    rows = 9
+    g = torch.Generator(device=DEV); g.manual_seed(V)
+    wide = inputs.zipf_gaussian_logits(rows, V + 13, seed=V, dtype=dtype, device=DEV)   # odd stride: every row another offset
+    logits = wide[:, start:start + V]
+    targets = inputs.uniform_targets(rows, V, seed=1, device=DEV)
+    targets[0], targets[1] = 0, V - 1
+    g_lp, g_en = torch.randn(rows, generator=g, device=DEV), torch.randn(rows, generator=g, device=DEV)
+    _check(e3, logits, targets, g_lp, g_en)                 # gradients elsewhere
+    lp, en = e3.e3_token_logp_entropy(logits, targets)
+    buf = torch.full((rows, V + 13), 7.0, dtype=dtype, device=DEV)
+    out = buf[:, start:start + V]                           # gradients at the logits' offsets
+    e3.e3_token_logp_entropy_backward(logits, targets, lp, en, g_lp, g_en, out=out)
+    ref = e3.e3_token_logp_entropy_backward(logits.contiguous(), targets, lp, en, g_lp, g_en)
+    assert torch.equal(out, ref) and torch.all(buf[:, :start] == 7.0) and torch.all(buf[:, start + V:] == 7.0)

@@ -104,3 +104,17 @@ def test_training_step_chain_objective_feeds_the_backward(e3):
                                              None, mask=mask.cpu().numpy())
     assert float(out[0]) == pytest.approx(J, abs=1e-5)
     assert np.abs(dz.cpu().numpy() - odz).max() < 1e-5
+
+
+@pytest.mark.parametrize("sizes,seq_len", [([3, 2], 2047), ([3, 2], 2049), ([4, 1, 2], 4100), ([1] * 2048, 3), ([1, 2] * 1025, 3)])
+def test_grpo_objective_at_the_edges_of_what_a_block_holds(e3, sizes, seq_len):
+    """Responses around the 2,048 tokens whose terms a block keeps, group counts around the 2,048 offsets it reads at a stroke."""
+    logp, logp_old, mask, adv, off = _case(seq_len, sizes, seq_len, seq_len // 2)
+    adv = np.where(adv == 0, np.float32(0.5), adv)          # (groups of one have no advantage: let them have a gradient)
+    t = lambda a: torch.from_numpy(a).to(DEV)
+    out, g = e3.e3_grpo_objective(t(logp), t(logp_old), t(adv), t(off), mask=t(mask).reshape(-1), clip_eps=0.2)
+    J, grad, frac = oracle.grpo_objective(logp, logp_old, mask, adv, off, 0.2)
+    assert float(out[0]) == pytest.approx(J, abs=1e-12) and float(out[1]) == pytest.approx(frac, abs=1e-12)
+    got = g.cpu().numpy().astype(np.float64)
+    assert np.array_equal(got == 0, grad == 0)
+    assert np.all(np.abs(got - grad) <= np.abs(grad) * 2.0 ** -23 + 1e-30)

@@ -49,7 +49,7 @@ GROUP = 8
 METRIC = "logit rows/s, fused sample+entropy, V=151,936"
 UNIT = "rows/s"
 # dram__bytes_read.sum + dram__bytes_write.sum of one e3_sample launch of this workload (ncu capture summarised in
-# profiles/rows_kernel_c2_ncu_full.txt and rows_kernel_sampler0_c2_ncu_full.txt), streaming kernel only.
+# profiles/rows_kernel_c2_ncu_full.txt and rows_kernel_sampler0_c2_ncu_full.txt).
 NCU_TRAFFIC_BYTES = {0: 161.7e6, 1: 160.0e6}
 WORKLOAD = "rollout decode step: 512 rows (64 prompts x 8 rollouts) x V=151,936 bf16, 256 decode steps"
 
@@ -342,8 +342,8 @@ def main():
     mean_host = torch.empty(2, dtype=torch.float64).pin_memory()
     sched = e3.make_sched(tau=1.0, V=V, t_anneal=288, t_max=480, eta=0.9)
     stream = torch.cuda.current_stream()
-    # kernels per step: the blocked sampler is two kernels per call; training pass 1 + 2 (fused sum); advantage 1
-    launches_per_step = DECODE_STEPS * (2 if args.sampler == 1 else 1) + 1 + 2 + 1
+    # kernels per step: one per sampling call; training pass 1 + 1 (fused sum); advantage 1
+    launches_per_step = DECODE_STEPS + 1 + 1 + 1
 
     def decode_loop(step_index):
         for d in range(DECODE_STEPS):
@@ -527,8 +527,7 @@ def main():
                        "rows_per_step": rows_per_step, "rows_per_step_with_masked": rows_per_step_all,
                        "value_with_masked_rows": world * rows_per_step_all * args.steps / (ms_total_max * 1e-3),
                        "e2e_steps": args.e2e_steps},
-            "roofline": {"bound": "hbm", "kernel": f"rows_kernel (e3_sample, sampler {args.sampler}, bf16)"
-                                                   + (" + block_sample_kernel" if args.sampler == 1 else ""),
+            "roofline": {"bound": "hbm", "kernel": f"rows_kernel (e3_sample, sampler {args.sampler}, bf16)",
                          "achieved": achieved, "peak": peak,
                          "peak_kind": peak_kind, "unit": "GB/s", "frac": achieved / peak,
                          "frac_of_measured_peak": achieved / peak, "frac_of_8TBs": achieved / 8000.0,

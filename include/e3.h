@@ -97,8 +97,8 @@ E3_API const char *e3_status_string(e3_status s);
 
 /* Bytes of device scratch a call uses for the given problem size.  For
  * E3_CALL_MASKED_MEAN_ENTROPY `rows` is the number of tokens n, for E3_CALL_GRPO_OBJECTIVE the number of
- * responses n_seq, for E3_CALL_SEQUENCE_MEAN_ENTROPY the number of sequences n_seq; V, dt are ignored for these.  E3_CALL_SAMPLE: 256 KiB for the partial states of cut rows plus,
- * for E3_SAMPLER_BLOCK, the per-lane sums the second kernel reads (about 1/32 of the bytes of the logits);
+ * responses n_seq, for E3_CALL_SEQUENCE_MEAN_ENTROPY the number of sequences n_seq; V, dt are ignored for these.  E3_CALL_SAMPLE: 256 KiB for the partial states of cut rows plus
+ * room for the sums of blocks (about 1/32 of the bytes of the logits), which the present kernels leave untouched;
  * E3_CALL_TOKEN_LOGP_ENTROPY: 256 KiB plus the partial sums of the fused mean entropy.
  * Scratch contents on entry never matter.  A workspace must not be shared by calls that can run
  * at the same time (different streams without ordering).  It must be 16-byte aligned. */
@@ -134,8 +134,7 @@ E3_API size_t e3_workspace_bytes(e3_call which, int64_t rows, int64_t V, e3_dtyp
  *   out_status  device int32 or NULL: status word, see the conventions above.
  *   workspace   device scratch of e3_workspace_bytes(E3_CALL_SAMPLE, ...) bytes.  It holds the partial states
  *               of rows that are split between thread blocks so that every block streams the same number
- *               of bytes, and what the two kernels of E3_SAMPLER_BLOCK hand to each other.  For the other
- *               samplers NULL (or fewer than 256 KiB) is accepted: rows are then never split, which costs
+ *               of bytes.  For samplers other than E3_SAMPLER_BLOCK NULL (or fewer than 256 KiB) is accepted: rows are then never split, which costs
  *               throughput when there are fewer than a few thousand rows.  E3_SAMPLER_BLOCK needs the full
  *               size (E3_ERR_WORKSPACE).
  * -inf logits are allowed (probability 0, never drawn).
@@ -159,8 +158,8 @@ E3_API e3_status e3_sample(const void *logits, e3_dtype dt, int64_t rows, int64_
  *               (Sec. 4.2) from the same call: out_ent_sum = sum_r mask[r] out_ent[r] accumulated in fp64 in
  *               the fixed order of e3_masked_mean_entropy, out_count = sum_r mask[r]; out_ent_sum / out_count
  *               equals that call's mean bit for bit.  Needs out_ent and the workspace
- *               (E3_ERR_INVALID_ARG / E3_ERR_WORKSPACE).  The reduction runs as two small kernels behind
- *               the row kernel, chained by programmatic dependent launch.
+ *               (E3_ERR_INVALID_ARG / E3_ERR_WORKSPACE).  The reduction runs as one small kernel (beyond 262,144
+ *               rows two) behind the row kernel, chained by programmatic dependent launch.
  *   workspace   e3_workspace_bytes(E3_CALL_TOKEN_LOGP_ENTROPY, rows, V, dt) bytes; NULL or fewer than
  *               256 KiB is accepted when the fused mean is not asked for (rows are then never split).
  * Other arguments as in e3_sample.

@@ -1,0 +1,90 @@
+"""The row kernel and the entropy mean at the edges of their splits, against the fp64 oracle (tolerances of `_compare`)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2505_18573_b200 import inputs
+from _compare import ATOL, assert_close, assert_tokens
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+@pytest.fixture(scope="module")
+def e3():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2505_18573_b200 import binding
+    binding.lib()
+    return binding
+
+
+def _check(e3, logits, temps, samplers=(0, 1), mask=None, workspace=None):
+    rows, V = logits.shape
+    z, t = inputs.to_oracle_array(logits), temps.cpu().numpy()
+    for sampler in samplers:
+        tok, lp, en = e3.e3_sample(logits, temps, 3, 1 << 34, 5, sampler, workspace=workspace)[:3]
+        ref = oracle.sample(z, t, 3, 1 << 34, 5, sampler)
+        tok = tok.cpu().numpy()
+        assert_tokens(f"V{V}r{rows}s{sampler}", tok, ref, sampler)
+        same = tok == ref.tok
+        assert_close("ent", en.cpu().numpy(), ref.ent, ATOL[logits.dtype])
+        assert_close("logp", lp.cpu().numpy()[same], ref.logp[same], ATOL[logits.dtype])
+    targets = inputs.uniform_targets(rows, V, seed=3, device=DEV)
+    lp, en = e3.e3_token_logp_entropy(logits, targets, mask=mask, temps=temps, workspace=workspace)[:2]
+    rlp, ren, _ = oracle.token_logp_entropy(z, targets.cpu().numpy(), mask=None if mask is None else mask.cpu().numpy(), temps=t)
+    assert_close("train.logp", lp.cpu().numpy(), rlp, ATOL[logits.dtype])
+    assert_close("train.ent", en.cpu().numpy(), ren, ATOL[logits.dtype])
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("rows, V", [
+    (5, 1024), (37, 2049), (149, 6145),   # one tile a row, a tile and an entry, three tiles and an entry
+    (17, 101000), (100, 101000),          # one strip per warp of 1 and of a few tiles
+    (290, 101000), (600, 33333)])         # strips of several waves; rows that begin anywhere
+def test_strip_lengths(e3, dtype, rows, V):
+    logits = inputs.zipf_gaussian_logits(rows, V, seed=rows, dtype=dtype, device=DEV)
+    _check(e3, logits, inputs.uniform_temps(rows, seed=V, device=DEV))
+
+
+@pytest.mark.parametrize("dtype, V", [(torch.bfloat16, 260001), (torch.bfloat16, 270001), (torch.float32, 300001)])
+def test_whole_rows_of_several_segments(e3, dtype, V):
+    """Without room for cut rows a block takes whole rows: more strips than half a ring of records, than a whole one."""
+    logits = inputs.zipf_gaussian_logits(3, V, seed=V, dtype=dtype, device=DEV)
+    tiny = torch.zeros(64, dtype=torch.uint8, device=DEV)
+    _check(e3, logits, inputs.uniform_temps(3, seed=1, device=DEV), samplers=(0,), workspace=tiny)
+
+
+def test_blocked_sampler_rows_longer_than_its_half_ring(e3):
+    rows, V = 140, 400001
+    logits = inputs.zipf_gaussian_logits(rows, V, seed=9, dtype=torch.float32, device=DEV)
+    _check(e3, logits, inputs.uniform_temps(rows, seed=2, device=DEV), samplers=(1,))
+
+
+@pytest.mark.parametrize("shift, rows", [(0, 1), (1, 15), (3, 16), (7, 17), (15, 500), (5, 12300)])
+def test_masks_that_begin_anywhere(e3, shift, rows):
+    g = torch.Generator(device="cpu").manual_seed(rows)
+    mask = (torch.rand(rows + shift, generator=g) < 0.6).to(torch.uint8).to(DEV)[shift:]
+    logits = inputs.zipf_gaussian_logits(rows, 2500, seed=rows, dtype=torch.bfloat16, device=DEV)
+    _check(e3, logits, inputs.uniform_temps(rows, seed=3, device=DEV), samplers=(), mask=mask)
+
+
+@pytest.mark.parametrize("std, temp", [(0.05, 1.0), (1.0, 1.0), (1.0, 3.0), (2.5, 1.0)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_token_sampler_on_flat_rows(e3, dtype, std, temp):
+    """Rows with many logits close to the largest, on both sides of the rule that passes over them for the first bound."""
+    g = torch.Generator(device=DEV); g.manual_seed(4)
+    logits = (torch.randn((65, 20000), generator=g, device=DEV) * std).to(dtype)
+    _check(e3, logits, torch.full((65,), temp, device=DEV), samplers=(0,))
+
+
+@pytest.mark.parametrize("n", [1, 1023, 32767, 32768, 32769, 65537, 262143, 262144, 262145, 300001])
+def test_mean_at_the_edges_of_a_cluster(e3, n):
+    g = torch.Generator(device="cpu").manual_seed(n)
+    ent = (torch.rand(n, generator=g) * 10).to(DEV)
+    mask = (torch.rand(n + 1, generator=g) < 0.7).to(torch.uint8).to(DEV)[1:]
+    for m in (mask, None):
+        out = e3.e3_masked_mean_entropy(ent, m)
+        mean, count = oracle.masked_mean_entropy(ent.cpu().numpy(), None if m is None else m.cpu().numpy())
+        assert float(out[1]) == count and float(out[0]) == pytest.approx(mean, rel=1e-12)

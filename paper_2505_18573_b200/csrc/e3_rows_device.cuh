@@ -28,7 +28,7 @@ constexpr float kMargin = 5.f;
 constexpr float kSoundZ = 128.f;
 constexpr float kSoundW = 1e30f;  // |sum 2^t t| of a sound tile stays far below (a -inf logit makes it NaN)
 
-enum : int { kErrValue = 1, kErrTimeout = 4 };
+enum : int { kErrValue = 1 };
 
 template <int DT>
 struct Fmt {

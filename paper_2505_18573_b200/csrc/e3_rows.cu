@@ -62,6 +62,7 @@
 // fp64 near a prefix boundary).
 #include "e3_rows.cuh"
 #include "e3_rows_device.cuh"
+#include "e3_rows_split.cuh"
 
 #include <atomic>
 #include <chrono>
@@ -70,30 +71,11 @@
 namespace e3 {
 namespace {
 
-constexpr int kWarps = 24;       // one CTA per SM: 80 registers a thread
 constexpr int kThreads = kWarps * 32;
 constexpr int kStages = 2;       // ring slots per warp
-constexpr int kRing = 256;       // most strips whose records the CTA keeps (RowsParams::ring of them are)
 constexpr int kMaxLive = 1024;   // rows of a CTA's run with a response mask (their numbers are kept in shared memory)
 constexpr int kQueueCap = 64;    // sampler 0: a push meets at most 31 entries and adds at most 32
-constexpr int kMaxBlocks = 512 * 8;  // sampler 1: blocks whose scores the CTA keeps (512 tiles)
-
-// The CTA's run of strips, numbered q = 0..len-1 in hand-out order: vocabulary order, except that the strips of the last row
-// come first when that row is cut.
-struct Run {
-  uint32_t q, r;        // all units = grid * q + r: CTA b starts at unit b*q + min(b, r)
-  int len;              // strips
-  uint32_t r0;          // row of the first strip (with a mask: its rank among the rows let through)
-  int n;                // rows touched
-  int lo0, hin;         // first strip within the first row; end strip within the last row (1..spr)
-  int head;             // strips of the last row that come first (0: none)
-};
-// Strip q of the run.
-struct Place {
-  int j;                // row: position in vocabulary order
-  int strip, lo, hi;    // strip within the row; strips of the row in this run
-  int q0;               // number of the row's first strip within the run
-};
+constexpr int kMaxBlocks = kBlockScoreTiles * 8;  // sampler 1: blocks whose scores the CTA keeps
 
 // An entry of sampler 0 that may win: vocabulary index (with kAnyByte: its coarse byte has not been looked at, else it is
 // 255) and logit.
@@ -136,7 +118,6 @@ struct LongPiece {
   int q0, turn;    // first strip; segments merged
   Piece state;
 };
-constexpr int kLong = 3;  // (such a piece is longer than half a ring: three of them at most are under way at a time)
 
 struct Smem {
   u64 full[kWarps][kStages];     // per warp and ring slot: the slot's tile has landed
@@ -192,50 +173,6 @@ __device__ __forceinline__ void post_best(u64 *bests, int seg, int enc) {
 __device__ __forceinline__ int read_best(const u64 *bests, int seg) {
   const u64 v = *reinterpret_cast<const volatile u64 *>(bests + (seg & (sm.p.ring - 1)));
   return (uint32_t)(v >> 32) == (uint32_t)(seg + 1) ? (int)((uint32_t)v ^ 0x80000000u) : enc_neg_inf();
-}
-
-// ---------------------------------------------------------------------------------------------
-// Work split
-// ---------------------------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t first_strip_of(const RowsParams &p, const Run &run, uint32_t b) {
-  return (b * run.q + (b < run.r ? b : run.r)) * (uint32_t)p.unit;
-}
-__device__ __forceinline__ int cta_of_strip(const RowsParams &p, const Run &run, uint32_t t) {
-  const uint32_t u = t / (uint32_t)p.unit, big = run.r * (run.q + 1);
-  return (int)(u < big ? u / (run.q + 1) : run.r + (u - big) / run.q);
-}
-// live: rows that are streamed (all, or those the mask lets through).
-__device__ __forceinline__ void set_run(const RowsParams &p, Run &run, uint32_t live) {
-  const uint32_t spr = (uint32_t)p.spr, unit = (uint32_t)p.unit, units = live * (spr / unit), b = blockIdx.x;
-  run.q = units / gridDim.x;
-  run.r = units - run.q * gridDim.x;
-  const uint32_t t0 = first_strip_of(p, run, b), len = (run.q + (b < run.r ? 1u : 0u)) * unit;
-  run.len = (int)len;
-  run.r0 = t0 / spr;
-  run.lo0 = (int)(t0 - run.r0 * spr);
-  const uint32_t end = t0 + len, row_last = len ? (end - 1u) / spr : run.r0;
-  run.hin = (int)(end - row_last * spr);
-  run.n = len ? (int)(row_last - run.r0) + 1 : 0;
-  run.head = run.n > 1 && run.hin < (int)spr ? run.hin : 0;
-}
-__device__ __forceinline__ Place place_of(const RowsParams &p, const Run &run, int q) {
-  Place w;
-  const bool head = q < run.head;
-  const int u = head ? q : q - run.head + run.lo0;  // strips from the start of the run's first row on (head: of its last)
-  int k = (int)((float)u * p.inv_spr);              // rows passed; off by one at most (u < 2^23)
-  int strip = u - k * p.spr;
-  if (strip >= p.spr) { strip -= p.spr; ++k; }
-  if (strip < 0) { strip += p.spr; --k; }
-  w.j = head ? run.n - 1 : k;
-  w.strip = strip;
-  w.lo = w.j == 0 ? run.lo0 : 0;
-  w.hi = w.j == run.n - 1 ? run.hin : p.spr;
-  w.q0 = q - (strip - w.lo);
-  return w;
-}
-// Strips of the segment that begins at w.
-__device__ __forceinline__ int segment_strips(const RowsParams &p, const Place &w) {
-  return w.hi - w.strip < p.ring / 2 ? w.hi - w.strip : p.ring / 2;
 }
 
 __device__ __forceinline__ const char *row_ptr(const RowsParams &p, uint32_t row) { return p.logits + (size_t)row * (size_t)p.row_bytes; }
@@ -427,7 +364,7 @@ __device__ __noinline__ bool finish_segment(int q, uint32_t row, float tau, floa
   __syncwarp();
   const bool single = w.hi - w.lo <= half, last = w.strip + n == w.hi;
   if (!single) {  // in the order of the segments (they are handed out in that order: the ones before are under way)
-    LongPiece &lp = sm.piece[(w.q0 / half) % kLong];
+    LongPiece &lp = sm.piece[long_piece_place(p, w)];
     const int turn = (w.strip - w.lo) / half;
     if (turn > 0) {
       const bool ok = bounded_wait([&] { return volatile_int(lp.q0) == w.q0 && volatile_int(lp.turn) == turn; });
@@ -623,7 +560,7 @@ __device__ __noinline__ void scan_mask(uint32_t *live_rows) {
     before += w < warp ? live_warp[w] : 0u;
     total += live_warp[w];
   }
-  if (tid == 0) set_run(p, sm.run, total);
+  if (tid == 0) set_run(p, sm.run, total, blockIdx.x, gridDim.x);
   __syncthreads();
   const uint32_t r0 = sm.run.r0, n = (uint32_t)sm.run.n;
   if (count > 0 && before < r0 + n && before + count > r0) {
@@ -687,7 +624,7 @@ __global__ void __launch_bounds__(kThreads, 1) rows_kernel(const __grid_constant
   if (tid == kThreads - 32) {
     sm.timeout = sm.exited = 0;
     sm.next = kWarps;  // (the first strips go to the warps by their numbers: a short run then loads the schedulers evenly)
-    if (p.mask == nullptr) set_run(p, sm.run, p.rows);
+    if (p.mask == nullptr) set_run(p, sm.run, p.rows, blockIdx.x, gridDim.x);
   }
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   __syncthreads();
@@ -736,16 +673,17 @@ __global__ void __launch_bounds__(kThreads, 1) rows_kernel(const __grid_constant
       dry = true;
       return;
     }
-    const int &freed = sm.freed[q & (p.ring - 1)];
-    if (volatile_int(freed) != q - p.ring + 1) {
+    const Place w = place_of(p, sm.run, q);
+    const int seg = segment_start(p, w);
+    auto free_places = [&] { return may_take(p, q, seg, [](int at) { return volatile_int(sm.freed[at]); }); };
+    if (!__all_sync(kAll, free_places())) {
       bool ok = false;
-      if (block) ok = bounded_wait([&] { return volatile_int(freed) == q - p.ring + 1; });
+      if (block) ok = bounded_wait(free_places);
       if (!__all_sync(kAll, ok)) {
         if (block) dry = true; else waiting = q;
         return;
       }
     }
-    const Place w = place_of(p, sm.run, q);
     const uint32_t row = live_rows ? live_rows[w.j] : sm.run.r0 + (uint32_t)w.j;
     const int tile = w.strip * p.strip_tiles;
     const char *const at = row_ptr(p, row) + (size_t)tile * kTileBytes;
@@ -762,12 +700,11 @@ __global__ void __launch_bounds__(kThreads, 1) rows_kernel(const __grid_constant
       skip = left - 1 - (int)((p.stall_src - at) / kTileBytes);
     if (strips > 0) load_aux(row, strips);  // (the first strip is taken before global memory may be read)
     if (lane == 0) {
-      const int half = p.ring / 2, first = (w.strip - w.lo) & ~(half - 1);  // of the segment, from the piece's first strip on
+      const int half = p.ring / 2, behind = w.q0 + w.hi - w.lo - seg;  // strips of the piece from the segment's first on
       StripMeta m;
-      m.q = q; m.tile = tile; m.row = row;
-      m.seg = w.q0 + first;
+      m.q = q; m.tile = tile; m.row = row; m.seg = seg;
       m.end = tile + left;
-      m.need = w.hi - w.lo - first < half ? w.hi - w.lo - first : half;
+      m.need = behind < half ? behind : half;
       sm.meta[warp][strips & 1] = m;
     }
     ++strips;
@@ -1155,22 +1092,6 @@ size_t pieces_bytes() { return (size_t)kMaxGrid * 2 * kPieceBytes; }
 // the SM's four schedulers.
 constexpr int64_t kStripsPerCta = 4;
 
-// Tiles per strip.  Strips of one length keep the warps of an SM in step, so that a run of a few strips per warp takes
-// whole waves: in a short run one strip per warp is all, the shortest that does it (151,936 bf16 entries a row, us for the lengths
-// below it, at it and behind it: statistics 256 rows 4 to 8 tiles 25.8, 26.8, 21.5, 21.9, 22.6, 512 rows 11 to 13 tiles 39.2,
-// 32.6, 33.6, 8 tiles 37.0; sampler 1 256 rows 35.2, 33.7, 27.5, 27.6, 28.5, 512 rows 45.9, 40.1, 40.2; sampler 0 512 rows 6, 12,
-// 13, 15 tiles 95, 87, 86, 94).  In a long run the waves dissolve: there a strip is as long as makes its own cost small (taking
-// it and handing in its record cost a warp about as many instructions as a tile's sums; for sampler 0 the first bound and the
-// last look at the queue cost twice that: 4,096 rows 12 tiles 537, 25 tiles 494), and for sampler 1 as short as the ring of block
-// scores asks for (4,096 rows 4, 6, 8 tiles 234, 266, 244; 1,024 rows 72, 75, 68).
-int strip_tiles(int64_t rows, int64_t tpr, int64_t ctas, int sampler) {
-  const int64_t per_warp = rows * tpr / ctas / kWarps, longest = sampler == 0 ? 25 : 13;
-  for (int64_t n = per_warp < 1 ? 1 : per_warp; n <= longest; ++n)
-    if (rows * ((tpr + n - 1) / n) <= ctas * kWarps) return (int)n;
-  if (sampler == 0) return 25;
-  return sampler == 1 && per_warp >= 32 ? 4 : 8;
-}
-
 template <int DT, int SAMPLER>
 cudaError_t launch_one(RowsParams p, int64_t rows, void *workspace, size_t workspace_bytes, cudaStream_t stream) {
   int64_t ctas = 0;
@@ -1184,9 +1105,7 @@ cudaError_t launch_one(RowsParams p, int64_t rows, void *workspace, size_t works
   p.spr = (int)spr;
   p.inv_spr = 1.0f / (float)spr;
   p.unit = can_cut ? 1 : (int)spr;
-  // the blocked sampler keeps the scores of 512 tiles' blocks
-  p.ring = kRing;
-  while (SAMPLER == 1 && p.ring * strip > 512) p.ring /= 2;
+  p.ring = ring_strips((int)strip, SAMPLER);
   p.ws_pieces = can_cut ? static_cast<unsigned char *>(workspace) : nullptr;
   p.wait_ns = kDefaultWaitNs;
   const long long stall = g_stall_tile.exchange(-1);  // (row * tpr + tile within the row)

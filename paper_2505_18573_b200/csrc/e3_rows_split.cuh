@@ -1,0 +1,129 @@
+// Work split of the row kernel: which strips a CTA takes, in which order they are handed out, and which places of
+// its rings they use.  Plain arithmetic without device state, so that the hand-out can be played through on the host
+// as well; P is RowsParams or anything with its fields spr, unit, ring and inv_spr.
+#pragma once
+#include <stdint.h>
+
+#ifdef __CUDACC__
+#define E3_SPLIT __host__ __device__ __forceinline__
+#else
+#define E3_SPLIT inline
+#endif
+
+namespace e3 {
+namespace {
+
+constexpr int kWarps = 24;           // one CTA per SM: 80 registers a thread
+constexpr int kRing = 256;           // most strips whose records the CTA keeps (RowsParams::ring of them are)
+constexpr int kBlockScoreTiles = 512;  // sampler 1: tiles whose block scores the CTA keeps
+
+// The CTA's run of strips, numbered q = 0..len-1 in hand-out order: vocabulary order, except that the strips of the last row
+// come first when that row is cut.
+struct Run {
+  uint32_t q, r;        // all units = grid * q + r: CTA b starts at unit b*q + min(b, r)
+  int len;              // strips
+  uint32_t r0;          // row of the first strip (with a mask: its rank among the rows let through)
+  int n;                // rows touched
+  int lo0, hin;         // first strip within the first row; end strip within the last row (1..spr)
+  int head;             // strips of the last row that come first (0: none)
+};
+// Strip q of the run.
+struct Place {
+  int j;                // row: position in vocabulary order
+  int strip, lo, hi;    // strip within the row; strips of the row in this run
+  int q0;               // number of the row's first strip within the run
+};
+
+template <class P>
+E3_SPLIT uint32_t first_strip_of(const P &p, const Run &run, uint32_t b) {
+  return (b * run.q + (b < run.r ? b : run.r)) * (uint32_t)p.unit;
+}
+template <class P>
+E3_SPLIT int cta_of_strip(const P &p, const Run &run, uint32_t t) {
+  const uint32_t u = t / (uint32_t)p.unit, big = run.r * (run.q + 1);
+  return (int)(u < big ? u / (run.q + 1) : run.r + (u - big) / run.q);
+}
+// The run of CTA b of `ctas`.  live: rows that are streamed (all, or those the mask lets through).
+template <class P>
+E3_SPLIT void set_run(const P &p, Run &run, uint32_t live, uint32_t b, uint32_t ctas) {
+  const uint32_t spr = (uint32_t)p.spr, unit = (uint32_t)p.unit, units = live * (spr / unit);
+  run.q = units / ctas;
+  run.r = units - run.q * ctas;
+  const uint32_t t0 = first_strip_of(p, run, b), len = (run.q + (b < run.r ? 1u : 0u)) * unit;
+  run.len = (int)len;
+  run.r0 = t0 / spr;
+  run.lo0 = (int)(t0 - run.r0 * spr);
+  const uint32_t end = t0 + len, row_last = len ? (end - 1u) / spr : run.r0;
+  run.hin = (int)(end - row_last * spr);
+  run.n = len ? (int)(row_last - run.r0) + 1 : 0;
+  run.head = run.n > 1 && run.hin < (int)spr ? run.hin : 0;
+}
+template <class P>
+E3_SPLIT Place place_of(const P &p, const Run &run, int q) {
+  Place w;
+  const bool head = q < run.head;
+  const int u = head ? q : q - run.head + run.lo0;  // strips from the start of the run's first row on (head: of its last)
+  int k = (int)((float)u * p.inv_spr);              // rows passed; off by one at most (u < 2^23)
+  int strip = u - k * p.spr;
+  if (strip >= p.spr) { strip -= p.spr; ++k; }
+  if (strip < 0) { strip += p.spr; --k; }
+  w.j = head ? run.n - 1 : k;
+  w.strip = strip;
+  w.lo = w.j == 0 ? run.lo0 : 0;
+  w.hi = w.j == run.n - 1 ? run.hin : p.spr;
+  w.q0 = q - (strip - w.lo);
+  return w;
+}
+// Strips of the segment that begins at w.
+template <class P>
+E3_SPLIT int segment_strips(const P &p, const Place &w) {
+  return w.hi - w.strip < p.ring / 2 ? w.hi - w.strip : p.ring / 2;
+}
+// Number (in the run) of the first strip of the segment that strip w belongs to.
+template <class P>
+E3_SPLIT int segment_start(const P &p, const Place &w) {
+  return w.q0 + ((w.strip - w.lo) & ~(p.ring / 2 - 1));
+}
+
+// Whether strip q of the segment that begins with strip number seg may be taken.  freed(place): 1 + number of the last strip
+// at this ring place whose record has been merged.  The segment's own state lies at the place of its first strip: while a short
+// segment one ring length before waits for a slow warp, that place is still in use although the strip's own may be free.
+// Segments are handed out in their order, so the oldest one that is not finished always finds its places free.
+template <class P, class F>
+E3_SPLIT bool may_take(const P &p, int q, int seg, F freed) {
+  return freed(q & (p.ring - 1)) == q - p.ring + 1 && freed(seg & (p.ring - 1)) == seg - p.ring + 1;
+}
+
+// State of a row piece of several segments, merged in their order: such a piece is longer than half a ring, three of them at
+// most are under way at a time.
+constexpr int kLong = 3;
+template <class P>
+E3_SPLIT int long_piece_place(const P &p, const Place &w) {
+  return w.q0 / (p.ring / 2) % kLong;
+}
+
+// ---- host: lengths of the strips
+// Tiles per strip.  Strips of one length keep the warps of an SM in step, so that a run of a few strips per warp takes
+// whole waves: in a short run one strip per warp is all, the shortest that does it (151,936 bf16 entries a row, us for the lengths
+// below it, at it and behind it: statistics 256 rows 4 to 8 tiles 25.8, 26.8, 21.5, 21.9, 22.6, 512 rows 11 to 13 tiles 39.2,
+// 32.6, 33.6, 8 tiles 37.0; sampler 1 256 rows 35.2, 33.7, 27.5, 27.6, 28.5, 512 rows 45.9, 40.1, 40.2; sampler 0 512 rows 6, 12,
+// 13, 15 tiles 95, 87, 86, 94).  In a long run the waves dissolve: there a strip is as long as makes its own cost small (taking
+// it and handing in its record cost a warp about as many instructions as a tile's sums; for sampler 0 the first bound and the
+// last look at the queue cost twice that: 4,096 rows 12 tiles 537, 25 tiles 494), and for sampler 1 as short as the ring of block
+// scores asks for (4,096 rows 4, 6, 8 tiles 234, 266, 244; 1,024 rows 72, 75, 68).
+inline int strip_tiles(int64_t rows, int64_t tpr, int64_t ctas, int sampler) {
+  const int64_t per_warp = rows * tpr / ctas / kWarps, longest = sampler == 0 ? 25 : 13;
+  for (int64_t n = per_warp < 1 ? 1 : per_warp; n <= longest; ++n)
+    if (rows * ((tpr + n - 1) / n) <= ctas * kWarps) return (int)n;
+  if (sampler == 0) return 25;
+  return sampler == 1 && per_warp >= 32 ? 4 : 8;
+}
+// Strips whose records a CTA keeps: sampler 1 keeps the scores of kBlockScoreTiles tiles' blocks.
+inline int ring_strips(int strip, int sampler) {
+  int ring = kRing;
+  while (sampler == 1 && ring * strip > kBlockScoreTiles) ring /= 2;
+  return ring;
+}
+
+}  // namespace
+}  // namespace e3

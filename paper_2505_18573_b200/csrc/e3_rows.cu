@@ -364,7 +364,7 @@ __device__ __noinline__ bool finish_segment(int q, uint32_t row, float tau, floa
   __syncwarp();
   const bool single = w.hi - w.lo <= half, last = w.strip + n == w.hi;
   if (!single) {  // in the order of the segments (they are handed out in that order: the ones before are under way)
-    LongPiece &lp = sm.piece[long_piece_place(p, w)];
+    LongPiece &lp = sm.piece[long_piece_place(w)];
     const int turn = (w.strip - w.lo) / half;
     if (turn > 0) {
       const bool ok = bounded_wait([&] { return volatile_int(lp.q0) == w.q0 && volatile_int(lp.turn) == turn; });

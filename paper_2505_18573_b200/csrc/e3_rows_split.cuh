@@ -94,12 +94,15 @@ E3_SPLIT bool may_take(const P &p, int q, int seg, F freed) {
   return freed(q & (p.ring - 1)) == q - p.ring + 1 && freed(seg & (p.ring - 1)) == seg - p.ring + 1;
 }
 
-// State of a row piece of several segments, merged in their order: such a piece is longer than half a ring, three of them at
-// most are under way at a time.
-constexpr int kLong = 3;
-template <class P>
-E3_SPLIT int long_piece_place(const P &p, const Place &w) {
-  return w.q0 / (p.ring / 2) % kLong;
+// A row piece of several segments (longer than half a ring) keeps a state in which they are merged in their order: one place for
+// the piece that the run begins with, three for the others in turn.  The places of rows j and j + 3 cannot meet: two whole rows,
+// so more than a ring of strips, lie between them.  While the last strip e of row j is not finished, strip e + ring cannot
+// be taken; it belongs to a full segment, whose records therefore stay, and so the strips one ring behind that segment cannot be
+// taken either.  These are more than there are warps (half a ring is at least 32 where a run is longer than a ring), and row
+// j + 3 has no full segment before them.
+constexpr int kLong = 4;
+E3_SPLIT int long_piece_place(const Place &w) {
+  return w.q0 == 0 && w.j > 0 ? kLong - 1 : w.j % (kLong - 1);
 }
 
 // ---- host: lengths of the strips

@@ -125,7 +125,7 @@ struct Cta {
         const int n = segment_strips(p, w), turn = (w.strip - w.lo) / half;
         const bool last = w.strip + n == w.hi;
         if (w.hi - w.lo > half) {
-          const int at = long_piece_place(p, w);
+          const int at = long_piece_place(w);
           if (at < 0 || at >= kLong) { fail("long piece number", q); return false; }
           if (turn > 0 && !(piece_owner[at] == w.q0 && piece_turn[at] == turn)) return false;
           if (turn == 0 && piece_live[at]) fail("long piece", q);

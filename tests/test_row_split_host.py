@@ -27,6 +27,14 @@ def test_state_of_a_segment_is_not_shared(model, rows, tiles, sampler, cta, slow
     _play(model, rows, tiles, sampler, 148, slow, cta, 1)
 
 
+@pytest.mark.parametrize("slow", [4, 400])
+@pytest.mark.parametrize("rows, tiles, sampler, cta", [
+    (300, 977, 1, 0), (1000, 600, 1, 0), (1000, 600, 1, 6),   # pieces of two to four half rings, one behind the other
+    (900, 1040, -1, 5), (700, 2100, -1, 3), (400, 6500, 0, 2)])
+def test_state_of_a_long_piece_is_not_shared(model, rows, tiles, sampler, cta, slow):
+    _play(model, rows, tiles, sampler, 148, slow, cta, 3)
+
+
 @pytest.mark.parametrize("rows, tiles, sampler", [(4096, 75, -1), (6144, 75, 0), (512, 75, 1), (2000, 125, 1), (900, 333, -1)])
 def test_every_block_finishes(model, rows, tiles, sampler):
     _play(model, rows, tiles, sampler, 148, 60, -1, 41)

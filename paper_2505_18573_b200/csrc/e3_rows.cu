@@ -788,6 +788,7 @@ __global__ void __launch_bounds__(kThreads, 1) rows_kernel(const __grid_constant
     bool more;
     do {
       float Zs = 0.f, Ws = 0.f, nRc = CUDART_INF_F, zmax = -CUDART_INF_F;  // the strip's sums; no reference yet
+      mode &= ~kCareful;  // (the form that sums a strip follows from the strip alone, not from the one before)
       const StripMeta &meta = sm.meta[warp][strip & 1];
       const int q = meta.q, first = meta.tile, end = meta.end;
       for (int tile = first; tile < end; ++tile) {
@@ -843,7 +844,7 @@ __global__ void __launch_bounds__(kThreads, 1) rows_kernel(const __grid_constant
                 if (summed || moved) break;
                 moved = true;
               }
-              if (!summed) mode |= kCareful;  // a -inf, a NaN, a +inf: the segment goes on carefully
+              if (!summed) mode |= kCareful;  // a -inf, a NaN, a +inf: the strip goes on carefully
               if (p.out_gap) zmax = fmaxf(zmax, warp_max(slice_max<DT>(B)));
             }
             if (!summed) {

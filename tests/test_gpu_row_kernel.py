@@ -62,6 +62,21 @@ def test_blocked_sampler_rows_longer_than_its_half_ring(e3):
     _check(e3, logits, inputs.uniform_temps(rows, seed=2, device=DEV), samplers=(1,))
 
 
+@pytest.mark.parametrize("dtype, rows, V", [(torch.float32, 148, 600000), (torch.bfloat16, 300, 700001)])
+def test_same_bits_with_entries_ruled_out(e3, dtype, rows, V):
+    """Logits of -inf here and there: the sums of a strip do not depend on which warp took it or what that warp summed before."""
+    g = torch.Generator(device=DEV); g.manual_seed(1)
+    logits = torch.randn((rows, V), generator=g, device=DEV).to(dtype)
+    logits.view(-1)[torch.randint(0, rows * V, (rows * 25,), generator=g, device=DEV)] = float("-inf")
+    temps, targets = torch.full((rows,), 0.9, device=DEV), torch.zeros(rows, dtype=torch.int32, device=DEV)
+    calls = (lambda: e3.e3_token_logp_entropy(logits, targets, temps=temps, want_gap=True),
+             lambda: e3.e3_sample(logits, temps, 1, 2), lambda: e3.e3_sample(logits, temps, 1, 2, sampler=e3.E3_SAMPLER_BLOCK))
+    for call in calls:
+        first = call()
+        for _ in range(12):
+            assert all(torch.equal(a, b) for a, b in zip(first, call()))
+
+
 @pytest.mark.parametrize("shift, rows", [(0, 1), (1, 15), (3, 16), (7, 17), (15, 500), (5, 12300)])
 def test_masks_that_begin_anywhere(e3, shift, rows):
     g = torch.Generator(device="cpu").manual_seed(rows)

@@ -222,17 +222,16 @@ Scratch scratch(PyObject *given, size_t need, at::Device device, cudaStream_t st
   return s;
 }
 
-// Runs a call of the library without the GIL (a full launch queue may make it wait).
+// Runs a call of the library without the GIL (a full launch queue may make it wait).  The call may throw (a tensor without
+// memory of its own, as under vmap): the GIL is back before that leaves.
 template <class F>
 e3_status launch(F call) {
-  PyThreadState *save = PyEval_SaveThread();
-  e3_status st;
-  {
-    std::lock_guard<std::mutex> hold(g_launch_lock);
-    st = call();
-  }
-  PyEval_RestoreThread(save);
-  return st;
+  struct Released {
+    PyThreadState *save = PyEval_SaveThread();
+    ~Released() { PyEval_RestoreThread(save); }
+  } released;
+  std::lock_guard<std::mutex> hold(g_launch_lock);
+  return call();
 }
 
 // ---- calls -----------------------------------------------------------------------------------------------------

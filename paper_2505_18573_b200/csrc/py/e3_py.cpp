@@ -8,14 +8,16 @@
 
 #include <ATen/cuda/EmptyTensor.h>
 #include <ATen/core/Tensor.h>
-#include <c10/cuda/CUDACachingAllocator.h>
-#include <c10/cuda/CUDAGraphsC10Utils.h>
+#include <c10/cuda/CUDAException.h>
+#include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <map>
+#include <memory>
 #include <mutex>
 #include <utility>
+#include <vector>
 
 #include "e3.h"
 #include "e3_internal.h"
@@ -168,21 +170,64 @@ PyObject *tuple_of(std::initializer_list<const Output *> outs) {
 }
 
 // ---- scratch ---------------------------------------------------------------------------------------------------
-// One buffer per (device, stream), grown on demand: calls that may overlap on the GPU must not share one.  At most kMostKept
-// of them; a buffer that is dropped goes back to torch's allocator, which is told that the stream may still use it.  While a
-// stream is being captured the buffer is made from the graph's own memory and not kept.  Callers that manage memory
+// One buffer per (device, stream), grown on demand: calls that may overlap on the GPU must not share one.  It is allocated on
+// the stream of the call, so that a buffer that is dropped (at most kMostKept are kept) is only ever used again in that stream's
+// order.  A call into a stream that is being captured gets a buffer of that capture instead (one per capture and stream), which
+// belongs to the graph: it lives until the graph and what has been instantiated from it are gone.  Callers that manage memory
 // themselves pass `workspace=` instead.
 constexpr size_t kMostKept = 64;
 using Key = std::pair<int, cudaStream_t>;
 std::map<Key, at::Tensor> *g_kept = new std::map<Key, at::Tensor>();  // used with the GIL held; never destroyed (torch may be gone by then)
 std::mutex g_launch_lock;                                             // a call's kernels go to the stream together
 
-void give_back(const Key &key, const at::Tensor &t) {
-  c10::cuda::CUDACachingAllocator::recordStream(
-      t.storage().data_ptr(),
-      key.second ? c10::cuda::getStreamFromExternal(key.second, static_cast<c10::DeviceIndex>(key.first))
-                 : c10::cuda::getDefaultCUDAStream(static_cast<c10::DeviceIndex>(key.first)));
+at::Tensor buffer_on(cudaStream_t stream, size_t bytes, at::Device device) {
+  const c10::cuda::CUDAStreamGuard guard(stream == nullptr || stream == cudaStreamLegacy
+                                             ? c10::cuda::getDefaultCUDAStream(device.index())
+                                             : c10::cuda::getStreamFromExternal(stream, device.index()));
+  return empty({static_cast<int64_t>(bytes < 16 ? 16 : bytes)}, at::kByte, device);
 }
+
+// Buffers of captures.
+using CaptureKey = std::pair<unsigned long long, cudaStream_t>;
+struct GraphBuffer {
+  CaptureKey key;
+  at::Tensor tensor;
+};
+std::map<CaptureKey, GraphBuffer *> *g_captured = new std::map<CaptureKey, GraphBuffer *>();  // the largest of each; with the GIL held
+std::mutex g_orphans_lock;
+std::vector<GraphBuffer *> *g_orphans = new std::vector<GraphBuffer *>();  // their graphs are gone
+// Called by the CUDA runtime, on a thread of its own that must not call it: the buffer waits for the next call.
+void CUDART_CB orphan(void *b) {
+  std::lock_guard<std::mutex> hold(g_orphans_lock);
+  g_orphans->push_back(static_cast<GraphBuffer *>(b));
+}
+void free_orphans() {
+  std::vector<GraphBuffer *> gone;
+  {
+    std::lock_guard<std::mutex> hold(g_orphans_lock);
+    gone.swap(*g_orphans);
+  }
+  for (GraphBuffer *b : gone) {
+    auto it = g_captured->find(b->key);
+    if (it != g_captured->end() && it->second == b) g_captured->erase(it);
+    delete b;
+  }
+}
+at::Tensor graph_buffer(unsigned long long id, cudaGraph_t graph, cudaStream_t stream, size_t need, at::Device device) {
+  const CaptureKey key(id, stream);
+  auto it = g_captured->find(key);
+  if (it != g_captured->end() && static_cast<size_t>(it->second->tensor.numel()) >= need) return it->second->tensor;
+  auto b = std::make_unique<GraphBuffer>(GraphBuffer{key, buffer_on(stream, need, device)});
+  cudaUserObject_t object;
+  C10_CUDA_CHECK(cudaUserObjectCreate(&object, b.get(), orphan, 1, cudaUserObjectNoDestructorSync));
+  GraphBuffer *const owned = b.release();
+  const cudaError_t e = cudaGraphRetainUserObject(graph, object, 1, cudaGraphUserObjectMove);
+  if (e != cudaSuccess) (void)cudaUserObjectRelease(object, 1);
+  C10_CUDA_CHECK(e);
+  (*g_captured)[key] = owned;
+  return owned->tensor;
+}
+
 struct Scratch {
   at::Tensor hold;
   void *data = nullptr;
@@ -195,23 +240,25 @@ Scratch scratch(PyObject *given, size_t need, at::Device device, cudaStream_t st
     s.bytes = static_cast<size_t>(t->numel()) * t->element_size();
     return s;
   }
-  const Key key(device.index(), stream);
-  const bool captured =
-      c10::cuda::currentStreamCaptureStatusMayInitCtx() != c10::cuda::CaptureStatus::None;
-  if (captured) {
-    s.hold = empty({static_cast<int64_t>(need < 16 ? 16 : need)}, at::kByte, device);
+  free_orphans();
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  cudaGraph_t graph = nullptr;
+  if (cudaStreamGetCaptureInfo_v2(stream, &status, &id, &graph, nullptr, nullptr) != cudaSuccess) {
+    (void)cudaGetLastError();  // (the launch will say what is wrong with the stream)
+    status = cudaStreamCaptureStatusNone;
+  }
+  if (status == cudaStreamCaptureStatusActive) {
+    s.hold = graph_buffer(id, graph, stream, need, device);
   } else {
+    const Key key(device.index(), stream);
     auto it = g_kept->find(key);
     if (it == g_kept->end() || static_cast<size_t>(it->second.numel()) < need) {
-      at::Tensor fresh = empty({static_cast<int64_t>(need < 16 ? 16 : need)}, at::kByte, device);
+      at::Tensor fresh = buffer_on(stream, need, device);
       if (it != g_kept->end()) {
-        give_back(key, it->second);
         it->second = std::move(fresh);
       } else {
-        if (g_kept->size() >= kMostKept) {
-          for (const auto &kv : *g_kept) give_back(kv.first, kv.second);
-          g_kept->clear();
-        }
+        if (g_kept->size() >= kMostKept) g_kept->clear();
         it = g_kept->emplace(key, std::move(fresh)).first;
       }
     }

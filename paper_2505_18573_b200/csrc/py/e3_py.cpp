@@ -8,6 +8,7 @@
 
 #include <ATen/cuda/EmptyTensor.h>
 #include <ATen/core/Tensor.h>
+#include <ATen/ops/empty_like.h>
 #include <c10/cuda/CUDAException.h>
 #include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
@@ -430,7 +431,11 @@ PyObject *group_advantage(PyObject *const *a) {
   const float eps = number(a[kEps]);
   const int unbiased = truth(a[kUnbiased]) ? 1 : 0;
   const bool own_adv = a[kAdv] == Py_None, own_flags = a[kFlags] == Py_None && truth(a[kWantFlags]);
-  const Output adv = output(a[kAdv], "out_adv", true, rewards.sizes(), at::kFloat, rewards.device());
+  Output adv = output(a[kAdv], "out_adv", rewards.is_contiguous(), rewards.sizes(), at::kFloat, rewards.device());
+  if (!adv.any) {  // groups go by the order in memory: permuted rewards give advantages permuted alike
+    adv.made = at::empty_like(rewards);
+    adv.any = true;
+  }
   const Output flags = output(a[kFlags], "out_flags", own_flags, {ng < 0 ? 0 : ng}, at::kByte, rewards.device());
   const cudaStream_t stream = stream_of(a[kStream]);
   check("e3_group_advantage", launch([&] {

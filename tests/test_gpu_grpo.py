@@ -118,3 +118,15 @@ def test_grpo_objective_at_the_edges_of_what_a_block_holds(e3, sizes, seq_len):
     got = g.cpu().numpy().astype(np.float64)
     assert np.array_equal(got == 0, grad == 0)
     assert np.all(np.abs(got - grad) <= np.abs(grad) * 2.0 ** -23 + 1e-30)
+
+
+def test_advantages_are_laid_out_like_the_rewards(e3):
+    """Groups go by the order in memory; permuted rewards give advantages with the same strides, as zeros_like does."""
+    rewards = torch.rand((6, 8), generator=torch.Generator().manual_seed(1)).to(DEV)
+    off = torch.tensor([3, 16, 40], dtype=torch.int64, device=DEV)  # entries before and behind the groups
+    want, flags = e3.e3_group_advantage(rewards, off)
+    turned, turned_flags = e3.e3_group_advantage(rewards.t(), off)
+    assert turned.shape == (8, 6) and turned.stride() == rewards.t().stride()
+    assert torch.equal(turned.t(), want) and torch.equal(flags, turned_flags)
+    adv, _ = e3.e3_group_advantage(torch.zeros(0, device=DEV), off[:1] * 0, out_flags=torch.zeros(0, dtype=torch.uint8, device=DEV))
+    assert adv.numel() == 0

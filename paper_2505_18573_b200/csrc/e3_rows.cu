@@ -36,9 +36,9 @@
 //
 // Numerics.  A strip's sums are Z = sum 2^t, W = sum 2^t * t with t = z*c - R*c and c = log2(e)/tau, two entries per
 // instruction (packed fp32).  R is the largest of a sample of 256 (bf16) or 128 (fp32) of the first tile's entries plus a
-// margin; one vote per tile checks its sums, and when an entry is far above R (or there is a NaN or an infinity) R moves up to
-// the tile's largest logit and the tile is summed again, and if that does not help in a careful form that masks -inf
-// entries and flags NaN and +inf.  R therefore stays close to the largest logit of the strip, which keeps W/Z small and the
+// margin; one vote per tile checks its sums, and when an entry is far above R (or there is a NaN or a +inf) R moves up to
+// the tile's largest logit and the tile is summed again; where there is a -inf it is summed with clamped entries, and if neither
+// helps in a careful form that flags NaN and +inf.  R therefore stays close to the largest logit of the strip, which keeps W/Z small and the
 // entropy free of cancellation.  Records merge associatively; the per-row result is formed in fp64:
 // H = ln Z - ln2 * W / Z,  ln p_tok = (z_tok*c - M) ln2 - ln Z, and, where the caller asks for it, the mean logit gap
 // beta sum p_i Delta_i = (z_max*c - M - W/Z) ln2 of App. A.
@@ -734,7 +734,7 @@ __global__ void __launch_bounds__(kThreads, 1) rows_kernel(const __grid_constant
     }
   };
 
-  enum : uint32_t { kGreedy = 1u, kUnusable = 2u, kCareful = 4u };
+  enum : uint32_t { kGreedy = 1u, kUnusable = 2u, kClamped = 4u };
   bool given_up = false;
   int strip = 0;  // strips summed
   // The warp's first strip is found before the kernel waits for the one before it in the stream (8 x 32,000 bf16: 9.0 us a
@@ -788,7 +788,6 @@ __global__ void __launch_bounds__(kThreads, 1) rows_kernel(const __grid_constant
     bool more;
     do {
       float Zs = 0.f, Ws = 0.f, nRc = CUDART_INF_F, zmax = -CUDART_INF_F;  // the strip's sums; no reference yet
-      mode &= ~kCareful;  // (the form that sums a strip follows from the strip alone, not from the one before)
       const StripMeta &meta = sm.meta[warp][strip & 1];
       const int q = meta.q, first = meta.tile, end = meta.end;
       for (int tile = first; tile < end; ++tile) {
@@ -813,56 +812,57 @@ __global__ void __launch_bounds__(kThreads, 1) rows_kernel(const __grid_constant
             float Z, W;
             float Zg[kG];
             bool summed = false;
-            // moves the strip's reference up to the logit R and rescales its sums; false when R c leaves the fp32 range
-            auto rebase = [&](float R) {
-              const float up = -R * c;
-              if (!(fabsf(up) < CUDART_INF_F)) return false;
-              if (up < nRc) {
-                const float d = up - nRc, f = nRc == CUDART_INF_F ? 0.f : ex2f(d);
-                Ws = f == 0.f ? 0.f : f * fmaf(d, Zs, Ws);
-                Zs = f == 0.f ? 0.f : f * Zs;
-                nRc = up;
-              }
-              return true;
-            };
-            if (n == F::kTileE && !(mode & kCareful)) {
-              if (nRc == CUDART_INF_F) {  // the reference from a sample: the lanes' first vectors
-                const uint4 v[1] = {lds128(B)};
-                const float up = -warp_max(vec_max<DT>(v)) * c - kMargin;
-                if (fabsf(up) < CUDART_INF_F) nRc = up;
-              }
-              bool moved = nRc == CUDART_INF_F;
-#pragma unroll 1
-              for (;;) {
-                if (moved) {
-                  const float R = warp_max(slice_max<DT>(B));
-                  if (R == -CUDART_INF_F || !rebase(R)) break;
+            // Out of line: what only few tiles need (see tile_slow).  The blocked sampler, whose short strips meet more of them, keeps
+            // all but the clamped sums in the loop.
+            constexpr bool kLean = SAMPLER != 1;
+            bool over = false;  // kLean: an entry far above the reference, or no reference yet
+            if (n == F::kTileE && !(mode & kClamped)) {
+              if (nRc == CUDART_INF_F) nRc = sample_reference<DT>(B, c);
+              // kClamped: a -inf (a NaN, a +inf).  The clamp changes no other sum, so that the warp may keep it through the segment and
+              // results still do not depend on which strips it takes.
+              if (kLean) {
+                over = nRc == CUDART_INF_F;
+                if (!over) {
+                  if (SAMPLER == 0) slice_sums_groups<DT>(B, c, nRc, Z, W, Zg);
+                  else slice_sums<DT>(B, c, nRc, Z, W);
+                  summed = !__any_sync(kAll, !(Z <= kSoundZ) || !(fabsf(W) <= kSoundW));
+                  if (!summed) {
+                    over = __any_sync(kAll, !(Z <= kSoundZ));
+                    if (!over) mode |= kClamped;
+                  } else if (p.out_gap) {
+                    zmax = fmaxf(zmax, warp_max(slice_max<DT>(B)));
+                  }
                 }
-                if (SAMPLER == 0) slice_sums_groups<DT>(B, c, nRc, Z, W, Zg);
-                else slice_sums<DT>(B, c, nRc, Z, W);
-                summed = !__any_sync(kAll, !(Z <= kSoundZ) || !(fabsf(W) <= kSoundW));
-                if (summed || moved) break;
-                moved = true;
+              } else {
+                bool moved = nRc == CUDART_INF_F;
+#pragma unroll 1
+                for (;;) {
+                  if (moved) {
+                    const float R = warp_max(slice_max<DT>(B));
+                    if (R == -CUDART_INF_F || !move_reference(R, c, nRc, Zs, Ws)) break;
+                  }
+                  slice_sums<DT>(B, c, nRc, Z, W);
+                  summed = !__any_sync(kAll, !(Z <= kSoundZ) || !(fabsf(W) <= kSoundW));
+                  if (summed || moved || !__any_sync(kAll, !(Z <= kSoundZ))) break;
+                  moved = true;
+                }
+                if (!summed) mode |= kClamped;
+                else if (p.out_gap) zmax = fmaxf(zmax, warp_max(slice_max<DT>(B)));
               }
-              if (!summed) mode |= kCareful;  // a -inf, a NaN, a +inf: the strip goes on carefully
-              if (p.out_gap) zmax = fmaxf(zmax, warp_max(slice_max<DT>(B)));
             }
-            if (!summed) {
-              const int nlane = n - lane * F::kLaneE;  // entries of the tile from the lane's first on (may be < 0)
-              const float R = warp_max(slice_max_careful<DT>(B, nlane, lane & 7));
-              zmax = fmaxf(zmax, R);
-              bool bad = R > -CUDART_INF_F && !rebase(R);
-              // without any reference (nothing finite so far) the sums must come out as zero
-              const bool none = nRc == CUDART_INF_F;
-              slice_sums_careful<DT>(B, nlane, lane & 7, c, none ? 0.f : nRc, Z, W, Zg);
-              bad |= !(Z <= kSoundZ) || !(fabsf(W) <= kSoundW) || (none && Z != 0.f);
-              if (__any_sync(kAll, bad)) {
-                err = kErrValue;
-                Z = W = 0.f;
+            if (!summed && (kLean || n == F::kTileE)) {
+              const SlowTile<DT> s = tile_slow<DT, SAMPLER == 0, kLean>(B, n, over, p.out_gap != nullptr, c, nRc, Zs, Ws);
+              Zs = s.Zs; Ws = s.Ws; nRc = s.nRc;
+              Z = s.Z; W = s.W;
+              zmax = fmaxf(zmax, s.zmax);
+              if (kLean && s.bad) err = kErrValue;
+              if (!kLean) summed = !s.bad;
+              if (SAMPLER == 0) {
 #pragma unroll
-                for (int j = 0; j < kG; ++j) Zg[j] = 0.f;
+                for (int j = 0; j < kG; ++j) Zg[j] = s.Zg[j];
               }
             }
+            if (!kLean && !summed && careful_tile<DT>(B, n, c, nRc, Zs, Ws, Z, W, Zg, zmax)) err = kErrValue;
             Zs += Z;
             Ws += W;
             if (SAMPLER == 0) {

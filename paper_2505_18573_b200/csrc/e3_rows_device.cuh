@@ -303,7 +303,7 @@ __device__ __forceinline__ void vec_sums(const uint4 &v, f2 c2, f2 nRc2, f2 &Za,
 
 // Sums of a whole slice: Z = sum 2^t, W = sum 2^t t.  A loop over the two halves of the slice: a body short enough for the
 // instruction cache.
-template <int DT>
+template <int DT, bool CLAMP = false>
 __device__ __forceinline__ void slice_sums(uint32_t B, float c, float nRc, float &Z, float &W) {
   const f2 c2 = pack2f(c, c), nRc2 = pack2f(nRc, nRc);
   f2 Za = pack2f(0.f, 0.f), Zb = Za, Wa = Za, Wb = Za;
@@ -313,13 +313,13 @@ __device__ __forceinline__ void slice_sums(uint32_t B, float c, float nRc, float
 #pragma unroll
     for (int i = 0; i < 4; ++i) v[i] = lds128((B ^ (uint32_t)(h * 64)) ^ (uint32_t)(i << 4));
 #pragma unroll
-    for (int i = 0; i < 4; ++i) vec_sums<DT, false>(v[i], c2, nRc2, Za, Zb, Wa, Wb);
+    for (int i = 0; i < 4; ++i) vec_sums<DT, CLAMP>(v[i], c2, nRc2, Za, Zb, Wa, Wb);
   }
   Z = sum2(add2(Za, Zb));
   W = sum2(add2(Wa, Wb));
 }
 // The same with the sum of 2^t of every group of 16 entries: Zg[j] belongs to group j xor ((lane mod 8) / vectors per group).
-template <int DT>
+template <int DT, bool CLAMP = false>
 __device__ __forceinline__ void slice_sums_groups(uint32_t B, float c, float nRc, float &Z, float &W, float (&Zg)[Fmt<DT>::kG]) {
   const f2 c2 = pack2f(c, c), nRc2 = pack2f(nRc, nRc);
   f2 Wa = pack2f(0.f, 0.f), Wb = Wa, Zt = Wa;
@@ -328,7 +328,7 @@ __device__ __forceinline__ void slice_sums_groups(uint32_t B, float c, float nRc
     f2 Za = pack2f(0.f, 0.f), Zb = Za;
 #pragma unroll
     for (int i = j * Fmt<DT>::kVG; i < (j + 1) * Fmt<DT>::kVG; ++i)
-      vec_sums<DT, false>(lds128(B ^ (uint32_t)(i << 4)), c2, nRc2, Za, Zb, Wa, Wb);
+      vec_sums<DT, CLAMP>(lds128(B ^ (uint32_t)(i << 4)), c2, nRc2, Za, Zb, Wa, Wb);
     Za = add2(Za, Zb);
     Zg[j] = sum2(Za);
     Zt = add2(Zt, Za);
@@ -350,6 +350,26 @@ __device__ __forceinline__ float slice_max(uint32_t B) {
   return m;
 }
 
+// -R c for a strip's reference R from a sample, the lanes' first vectors; +inf: none (no finite entry there).
+template <int DT>
+__device__ __forceinline__ float sample_reference(uint32_t B, float c) {
+  const uint4 v[1] = {lds128(B)};
+  const float up = -warp_max(vec_max<DT>(v)) * c - kMargin;
+  return fabsf(up) < CUDART_INF_F ? up : CUDART_INF_F;
+}
+// Moves a strip's reference up (nRc down) to the logit R and rescales its sums; false when R c leaves the fp32 range.
+__device__ __forceinline__ bool move_reference(float R, float c, float &nRc, float &Zs, float &Ws) {
+  const float up = -R * c;
+  if (!(fabsf(up) < CUDART_INF_F)) return false;
+  if (up < nRc) {
+    const float d = up - nRc, f = nRc == CUDART_INF_F ? 0.f : ex2f(d);
+    Ws = f == 0.f ? 0.f : f * fmaf(d, Zs, Ws);
+    Zs = f == 0.f ? 0.f : f * Zs;
+    nRc = up;
+  }
+  return true;
+}
+
 // The vector number i (counted from 0 to 7 in vocabulary order) of a slice of which the first nlane entries are valid:
 // the others become -inf.
 template <int DT>
@@ -367,9 +387,9 @@ __device__ __forceinline__ uint4 mask_vec(const uint4 &v, int nlane, int i) {
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// The careful form, for a tile that lies only partly inside the row and for one whose sums stay out of range with its
-// largest logit as reference (a -inf, a NaN, a +inf): entries are masked and clamped.  One vector per step, so that the code that
-// few tiles run stays short.
+// The careful form, for a tile that lies only partly inside the row and for one whose sums stay out of range clamped and with its
+// largest logit as reference (a NaN, a +inf): entries are masked and clamped.  One vector per step, so that the code that few
+// tiles run stays short.
 template <int DT>
 __device__ __forceinline__ float slice_max_careful(uint32_t B, int nlane, int r8) {
   float m = -CUDART_INF_F;
@@ -398,6 +418,72 @@ __device__ __forceinline__ void slice_sums_careful(uint32_t B, int nlane, int r8
     for (int j = 0; j < Fmt<DT>::kG; ++j) Zg[j] += i / Fmt<DT>::kVG == j ? z : 0.f;
   }
   W = sum2(add2(Wa, Wb));
+}
+
+// Sums of a tile in the careful form; the strip's reference moves up to the tile's largest logit first (zmax takes it in).  True: a
+// NaN, a +inf, or numbers outside the fp32 range (the sums are 0 then).
+template <int DT>
+__device__ __forceinline__ bool careful_tile(uint32_t B, int n, float c, float &nRc, float &Zs, float &Ws, float &Z, float &W,
+                                             float (&Zg)[Fmt<DT>::kG], float &zmax) {
+  const int lane = threadIdx.x & 31, nlane = n - lane * Fmt<DT>::kLaneE;  // entries from the lane's first on (may be < 0)
+  const float R = warp_max(slice_max_careful<DT>(B, nlane, lane & 7));
+  zmax = fmaxf(zmax, R);
+  bool bad = R > -CUDART_INF_F && !move_reference(R, c, nRc, Zs, Ws);
+  // without any reference (nothing finite so far) the sums must come out as zero
+  const bool none = nRc == CUDART_INF_F;
+  slice_sums_careful<DT>(B, nlane, lane & 7, c, none ? 0.f : nRc, Z, W, Zg);
+  bad |= !(Z <= kSoundZ) || !(fabsf(W) <= kSoundW) || (none && Z != 0.f);
+  bad = __any_sync(0xffffffffu, bad);
+  if (bad) {
+    Z = W = 0.f;
+#pragma unroll
+    for (int j = 0; j < Fmt<DT>::kG; ++j) Zg[j] = 0.f;
+  }
+  return bad;
+}
+
+// Sums of a tile that the streaming loop's plain form does not give: with a -inf, a NaN or a +inf, and with CAREFUL one that lies
+// only partly inside the row or has an entry far above the strip's reference (`over`: the reference moves first).  A full tile is
+// summed with clamped entries in the plain form's order, its reference following the same steps: the same bits where no
+// entry is that low.
+// Out of line: the streaming loop stays short (bound by issue and instruction fetch).  us with it inside the loop, with the clamped
+// sums alone out of line, and with all of it: statistics 4,096 x 151,936 bf16 211, 208, 204, token sampler 512 rows 88.5, 88.5,
+// 85.5, 8 rows 28.4, 28.9, 27.0, blocked sampler 4,096 rows 252, 247, 262.  A tenth of the logits -inf, 2,048 rows, one
+// vector at a time before and now: statistics 222 and 125, blocked 248 and 161, token sampler 421 and 317.
+template <int DT>
+struct SlowTile {
+  float Zs, Ws, nRc;  // the strip's sums and reference, moved
+  float Z, W, zmax;
+  float Zg[Fmt<DT>::kG];
+  bool bad;           // not summed: a NaN, a +inf, or numbers outside the fp32 range
+};
+template <int DT, bool GROUPS, bool CAREFUL>
+__device__ __noinline__ SlowTile<DT> tile_slow(uint32_t B, int n, bool over, bool want_max, float c, float nRc, float Zs, float Ws) {
+  SlowTile<DT> s;
+  s.zmax = -CUDART_INF_F;
+  s.bad = true;
+  if (!CAREFUL || n == Fmt<DT>::kTileE) {
+    if (nRc == CUDART_INF_F && !over) nRc = sample_reference<DT>(B, c);
+    bool moved = over || nRc == CUDART_INF_F;
+#pragma unroll 1
+    for (;;) {
+      bool none = false;  // no finite entry so far: the sums must come out as 0
+      if (moved) {
+        const float R = warp_max(slice_max<DT>(B));
+        none = R == -CUDART_INF_F && nRc == CUDART_INF_F;
+        if (!none && !move_reference(R, c, nRc, Zs, Ws)) break;
+      }
+      if (GROUPS) slice_sums_groups<DT, true>(B, c, none ? 0.f : nRc, s.Z, s.W, s.Zg);
+      else slice_sums<DT, true>(B, c, none ? 0.f : nRc, s.Z, s.W);
+      s.bad = __any_sync(0xffffffffu, !(s.Z <= (none ? 0.f : kSoundZ)) || !(fabsf(s.W) <= kSoundW));
+      if (!s.bad || moved) break;
+      moved = true;
+    }
+    if (!s.bad && want_max) s.zmax = warp_max(slice_max<DT>(B));
+  }
+  if (CAREFUL && s.bad) s.bad = careful_tile<DT>(B, n, c, nRc, Zs, Ws, s.Z, s.W, s.Zg, s.zmax);
+  s.Zs = Zs; s.Ws = Ws; s.nRc = nRc;
+  return s;
 }
 
 // A tile that begins `a` bytes (1..15) behind a 16-byte boundary was copied from that boundary on: moves it down by a

@@ -77,6 +77,27 @@ def test_same_bits_with_entries_ruled_out(e3, dtype, rows, V):
             assert all(torch.equal(a, b) for a, b in zip(first, call()))
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_entries_ruled_out(e3, dtype):
+    """-inf logits in whole tiles, in parts of them, with a logit far above the others, with a NaN or a +inf (the row reads NaN)."""
+    V, rows = 41003, 12
+    g = torch.Generator(device=DEV); g.manual_seed(6)
+    z = torch.randn((rows, V), generator=g, device=DEV)
+    drop = torch.rand((rows, V), generator=g, device=DEV) < 0.1
+    z[0][drop[0]] = float("-inf")
+    z[1, V // 2:] = float("-inf"); z[2, :V // 2] = float("-inf")
+    z[3, :] = float("-inf"); z[3, 7777] = 0.5
+    z[4][~drop[4]] = float("-inf")
+    z[5][drop[5]] = float("-inf"); z[5, 30000] = 60.0
+    z[6][drop[6]] = float("-inf"); z[6, 12345] = float("nan")
+    z[7][drop[7]] = float("-inf"); z[7, 12345] = float("inf")
+    z[8, 4096:8192] = float("-inf"); z[8, 5000] = float("nan")
+    z[9, 4096:8192] = float("-inf"); z[9, 5000] = float("inf")
+    z[10, 100:] = float("-inf")
+    z[11, 20000] = -3.0e38
+    _check(e3, z.to(dtype), inputs.uniform_temps(rows, seed=4, device=DEV))
+
+
 @pytest.mark.parametrize("shift, rows", [(0, 1), (1, 15), (3, 16), (7, 17), (15, 500), (5, 12300)])
 def test_masks_that_begin_anywhere(e3, shift, rows):
     g = torch.Generator(device="cpu").manual_seed(rows)

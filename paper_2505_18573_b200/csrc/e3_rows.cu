@@ -1099,7 +1099,7 @@ cudaError_t launch_one(RowsParams p, int64_t rows, void *workspace, size_t works
   cudaError_t e = resident_ctas<DT, SAMPLER>(ctas);
   if (e != cudaSuccess) return e;
   const int64_t tpr = ((int64_t)p.V + Fmt<DT>::kTileE - 1) / Fmt<DT>::kTileE;
-  const int64_t strip = strip_tiles(rows, tpr, ctas, SAMPLER), spr = (tpr + strip - 1) / strip;
+  const int64_t strip = strip_tiles(rows, tpr, ctas, SAMPLER, Fmt<DT>::kTileE), spr = (tpr + strip - 1) / strip;
   const bool can_cut = workspace != nullptr && workspace_bytes >= pieces_bytes();
   p.tpr = (int)tpr;
   p.strip_tiles = (int)strip;

@@ -177,7 +177,7 @@ int main(int argc, char **argv) {
   if (argc != 8) return 2;
   const long rows = atol(argv[1]), tpr = atol(argv[2]);
   const int sampler = atoi(argv[3]), ctas = atoi(argv[4]), slow = atoi(argv[5]), cta = atoi(argv[6]), apart = atoi(argv[7]);
-  const int strip = strip_tiles(rows, tpr, ctas, sampler);
+  const int strip = strip_tiles(rows, tpr, ctas, sampler, 2048);
   Split p;
   p.spr = (int)((tpr + strip - 1) / strip);
   p.unit = 1;

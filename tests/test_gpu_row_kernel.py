@@ -48,6 +48,13 @@ def test_strip_lengths(e3, dtype, rows, V):
     _check(e3, logits, inputs.uniform_temps(rows, seed=V, device=DEV))
 
 
+@pytest.mark.parametrize("dtype, rows, V", [(torch.bfloat16, 1790, 18001),   # one strip in a hundred more than warps, a short one
+                                            (torch.float32, 300, 252000)])   # one strip per warp of more tiles than bf16 has
+def test_strips_of_the_statistics(e3, dtype, rows, V):
+    logits = inputs.zipf_gaussian_logits(rows, V, seed=rows, dtype=dtype, device=DEV)
+    _check(e3, logits, inputs.uniform_temps(rows, seed=V, device=DEV), samplers=())
+
+
 @pytest.mark.parametrize("dtype, V", [(torch.bfloat16, 260001), (torch.bfloat16, 270001), (torch.float32, 300001)])
 def test_whole_rows_of_several_segments(e3, dtype, V):
     """Without room for cut rows a block takes whole rows: more strips than half a ring of records, than a whole one."""

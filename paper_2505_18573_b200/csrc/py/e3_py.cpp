@@ -301,7 +301,10 @@ PyObject *sample(PyObject *const *a) {
   const Output ent = output(a[kEnt], "out_ent", truth(a[kWantEnt]), {l.rows}, at::kFloat, l.device);
   const Output gap = output(a[kGap], "out_gap", truth(a[kWantGap]), {l.rows}, at::kFloat, l.device);
   const cudaStream_t stream = stream_of(a[kStream]);
-  const Scratch ws = scratch(a[kWorkspace], e3_workspace_bytes(E3_CALL_SAMPLE, l.rows, l.V, l.dt), l.device, stream);
+  // the blocked sampler asks for its full size; for the others the room for cut rows is enough (that of a training pass of no rows)
+  const size_t need = sampler == E3_SAMPLER_BLOCK ? e3_workspace_bytes(E3_CALL_SAMPLE, l.rows, l.V, l.dt)
+                                                  : e3_workspace_bytes(E3_CALL_TOKEN_LOGP_ENTROPY, 0, l.V, l.dt);
+  const Scratch ws = scratch(a[kWorkspace], need, l.device, stream);
   check("e3_sample", launch([&] {
           return e3_sample(l.data, l.dt, l.rows, l.V, l.stride, pointer<float>(temps), seed, counter, row_base, sampler,
                            tok.data<int32_t>(), logp.data<float>(), ent.data<float>(), gap.data<float>(),

@@ -30,7 +30,7 @@ class _Calls:
         self.need = e3.e3_workspace_bytes(e3.E3_CALL_SAMPLE, rows, V, e3.E3_F32)
 
     def __call__(self, stream):
-        self.e3.e3_sample(self.logits, self.temps, 3, 4, out_tok=self.tok, out_logp=self.logp, out_ent=self.ent, stream=stream)
+        self.e3.e3_sample(self.logits, self.temps, 3, 4, sampler=self.e3.E3_SAMPLER_BLOCK, out_tok=self.tok, out_logp=self.logp, out_ent=self.ent, stream=stream)
 
     def results(self):
         torch.cuda.synchronize()
@@ -126,6 +126,17 @@ def test_memory_of_dropped_graphs_comes_back(e3):
             break
         time.sleep(0.02)
     assert torch.cuda.memory_allocated() <= base
+
+
+def test_the_token_sampler_keeps_room_for_cut_rows_alone(e3):
+    logits = torch.zeros((512, 151936), dtype=torch.bfloat16, device=DEV)
+    temps, side = torch.ones(512, device=DEV), torch.cuda.Stream()
+    outs = e3.e3_sample(logits, temps, 1, 2)
+    torch.cuda.synchronize()
+    base = torch.cuda.memory_allocated()
+    e3.e3_sample(logits, temps, 1, 2, out_tok=outs[0], out_logp=outs[1], out_ent=outs[2], stream=side)
+    torch.cuda.synchronize()
+    assert torch.cuda.memory_allocated() - base < 1 << 20
 
 
 def test_many_streams_share_nothing(e3):

@@ -42,7 +42,8 @@ def _check(e3, logits, temps, samplers=(0, 1), mask=None, workspace=None):
 @pytest.mark.parametrize("rows, V", [
     (5, 1024), (37, 2049), (149, 6145),   # one tile a row, a tile and an entry, three tiles and an entry
     (17, 101000), (100, 101000),          # one strip per warp of 1 and of a few tiles
-    (290, 101000), (600, 33333)])         # strips of several waves; rows that begin anywhere
+    (290, 101000), (600, 33333),          # ... of a few tiles more, most warps busy; rows that begin anywhere
+    (700, 65001)])                        # strips of 8 tiles and more than one per warp
 def test_strip_lengths(e3, dtype, rows, V):
     logits = inputs.zipf_gaussian_logits(rows, V, seed=rows, dtype=dtype, device=DEV)
     _check(e3, logits, inputs.uniform_temps(rows, seed=V, device=DEV))
@@ -55,6 +56,38 @@ def test_strips_of_the_statistics(e3, dtype, rows, V):
     _check(e3, logits, inputs.uniform_temps(rows, seed=V, device=DEV), samplers=())
 
 
+@pytest.mark.parametrize("sampler, dtype, rows, V", [
+    (None, torch.bfloat16, 9000, 70001), (None, torch.bfloat16, 600, 1200001),  # rows of 5 strips, of several segments
+    (1, torch.bfloat16, 2500, 70001), (1, torch.bfloat16, 4000, 70001),         # strips of 8 tiles, of 4
+    (1, torch.float32, 400, 300001), (1, torch.float32, 200, 700001),           # pieces of two segments, of three
+    (0, torch.bfloat16, 16000, 70001)])
+def test_runs_longer_than_the_ring(e3, sampler, dtype, rows, V):
+    """More strips in a block's run than it keeps records of, rows that begin anywhere: the same as in batches of a few rows, where
+    no warp takes a second strip."""
+    g = torch.Generator(device=DEV); g.manual_seed(rows)
+    logits = torch.empty((rows, V), dtype=dtype, device=DEV)
+    for lo in range(0, rows, 500):
+        logits[lo:lo + 500] = torch.randn((min(500, rows - lo), V), generator=g, device=DEV) * 2.5
+    temps, targets = inputs.uniform_temps(rows, seed=V, device=DEV), inputs.uniform_targets(rows, V, seed=3, device=DEV)
+
+    def call(lo, hi):
+        if sampler is None:
+            return e3.e3_token_logp_entropy(logits[lo:hi], targets[lo:hi], temps=temps[lo:hi])
+        return e3.e3_sample(logits[lo:hi], temps[lo:hi], 7, 8, lo, sampler)
+    got = call(0, rows)
+    step = max(1, min(rows, 40 * 70001 // V))
+    parts = [torch.cat(t) for t in zip(*(call(lo, min(lo + step, rows)) for lo in range(0, rows, step)))]
+    if sampler is not None:
+        assert torch.equal(got[0], parts[0])
+    for a, b in zip(got[-2:], parts[-2:]):  # logp and ent: fp32 sums in another order
+        assert_close("small batches", a.cpu().numpy(), b.cpu().numpy(), 2e-5)
+    some = torch.arange(0, rows, max(1, rows // 9), device=DEV)
+    p = torch.log_softmax(logits[some].double() / temps[some, None].double(), 1)
+    assert_close("ent", got[-1][some].cpu().numpy(), -(p.exp() * p).sum(1).cpu().numpy(), ATOL[torch.float32])
+    at = (targets if sampler is None else got[0])[some].long()
+    assert_close("logp", got[-2][some].cpu().numpy(), p.gather(1, at[:, None])[:, 0].cpu().numpy(), ATOL[torch.float32])
+
+
 @pytest.mark.parametrize("dtype, V", [(torch.bfloat16, 260001), (torch.bfloat16, 270001), (torch.float32, 300001)])
 def test_whole_rows_of_several_segments(e3, dtype, V):
     """Without room for cut rows a block takes whole rows: more strips than half a ring of records, than a whole one."""
@@ -64,6 +97,7 @@ def test_whole_rows_of_several_segments(e3, dtype, V):
 
 
 def test_blocked_sampler_rows_longer_than_its_half_ring(e3):
+    """Rows of several segments in a run that still fits the ring."""
     rows, V = 140, 400001
     logits = inputs.zipf_gaussian_logits(rows, V, seed=9, dtype=torch.float32, device=DEV)
     _check(e3, logits, inputs.uniform_temps(rows, seed=2, device=DEV), samplers=(1,))

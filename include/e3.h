@@ -110,8 +110,9 @@ E3_API size_t e3_workspace_bytes(e3_call which, int64_t rows, int64_t V, e3_dtyp
  * drawn from p with the Gumbel-max construction; out_logp[r] = ln p[out_tok[r]].
  *
  *   logits      device, row-major [rows, V], element type `dt`, row r starts at
- *               element r * row_stride (row_stride >= V, in elements).  Rows whose
- *               start is 16-byte aligned take the vectorised path; others a slower one.
+ *               element r * row_stride (row_stride >= V, in elements).  Rows
+ *               may begin anywhere; those that do not begin on a 16-byte boundary cost one more move of
+ *               their tiles in shared memory.
  *   temps       device float [rows].  tau > 0 samples; tau == 0 is greedy
  *               (lowest-index arg-max, logp = 0, ent = 0); tau < 0, NaN, inf mark the row invalid.
  *   seed, counter, row_base
@@ -130,7 +131,7 @@ E3_API size_t e3_workspace_bytes(e3_call which, int64_t rows, int64_t V, e3_dtyp
  *   out_tok     device int32 [rows], required.   out_logp, out_ent: device float [rows], each may be NULL.
  *   out_gap     device float [rows] or NULL: the mean logit gap of App. A in units of tau,
  *               beta sum_i p_i Delta_i with Delta_i = z_max - z_i (so that H = ln sum_i exp(-beta Delta_i) + gap);
- *               0 for greedy rows.  Asking for it selects a kernel variant that also tracks z_max.
+ *               0 for greedy rows.  Asking for it makes the kernel track z_max too (a few per cent more time).
  *   out_status  device int32 or NULL: status word, see the conventions above.
  *   workspace   device scratch of e3_workspace_bytes(E3_CALL_SAMPLE, ...) bytes.  It holds the partial states
  *               of rows that are split between thread blocks so that every block streams the same number

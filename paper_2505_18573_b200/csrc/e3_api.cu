@@ -119,8 +119,8 @@ extern "C" e3_status e3_token_logp_entropy(const void *logits, e3_dtype dt, int6
   p.slack_scale = 1.f;
   cudaError_t e = e3::launch_rows(p, rows, static_cast<int>(dt), -1, workspace,
                                   workspace_bytes < token_mean_offset() ? workspace_bytes : token_mean_offset(), cs);
-  // The fused mean entropy: the two reduction kernels of e3_masked_mean_entropy behind the row kernel, chained by
-  // programmatic dependent launch; the same blocks add the same values in the same order.
+  // The fused mean entropy: the reduction of e3_masked_mean_entropy (one kernel, two beyond 262,144 rows) behind the row kernel,
+  // chained by programmatic dependent launch; the same blocks add the same values in the same order.
   if (e == cudaSuccess && fused_mean)
     e = e3::launch_masked_mean(out_ent, mask, rows, out_ent_sum, out_count,
                                static_cast<unsigned char *>(workspace) + token_mean_offset(), true, cs);

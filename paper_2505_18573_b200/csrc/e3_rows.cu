@@ -175,69 +175,9 @@ __device__ __forceinline__ int read_best(const u64 *bests, int seg) {
   return (uint32_t)(v >> 32) == (uint32_t)(seg + 1) ? (int)((uint32_t)v ^ 0x80000000u) : enc_neg_inf();
 }
 
-__device__ __forceinline__ const char *row_ptr(const RowsParams &p, uint32_t row) { return p.logits + (size_t)row * (size_t)p.row_bytes; }
-
 // ---------------------------------------------------------------------------------------------
 // Row results
 // ---------------------------------------------------------------------------------------------
-struct RowInfo {
-  float c;
-  bool greedy;
-};
-
-// One thread, fp64.  zt: logit of the token whose log-probability is wanted.
-__device__ __forceinline__ void finish_row(const RowsParams &p, uint32_t row, const RowInfo &ri, float Mf, float Zf,
-                                           float Wf, float zmax, int idx, int err, bool have_zt, float zt) {
-  const double M = Mf, Z = Zf, W = Wf;
-  const bool sample = p.mode == kModeSample;
-  int tok = -1;
-  float logp = CUDART_NAN_F, ent = CUDART_NAN_F, gap = CUDART_NAN_F;
-  if (ri.greedy) {
-    if (err == 0 && idx >= 0) { tok = idx; logp = 0.f; ent = 0.f; gap = 0.f; }
-  } else if (err == 0 && Z > 0.0) {
-    const double lnZ = log(Z), mean = W / Z;
-    ent = (float)(lnZ - kLn2 * mean);
-    // sum p_i (s_max - s_i) with s = z/tau: the mean of s is (M + W/Z) ln2
-    gap = (float)(((double)zmax * (double)ri.c - M - mean) * kLn2);
-    if (sample) tok = idx;
-    if (have_zt) logp = (float)(((double)zt * (double)ri.c - M) * kLn2 - lnZ);
-  }
-  if (p.out_ent) p.out_ent[row] = ent;
-  if (p.out_gap) p.out_gap[row] = gap;
-  if (sample) p.out_tok[row] = tok;
-  if (p.out_logp) p.out_logp[row] = logp;
-}
-
-// A row without a result: masked out (v = 0) or given up on because a wait ran out (v = NaN).
-__device__ __forceinline__ void write_plain(const RowsParams &p, uint32_t row, float v) {
-  if (p.mode == kModeSample) p.out_tok[row] = -1;
-  if (p.out_logp) p.out_logp[row] = v;
-  if (p.out_ent) p.out_ent[row] = v;
-  if (p.out_gap) p.out_gap[row] = v;
-}
-
-__device__ __forceinline__ void piece_reset(Piece &pc) {
-  pc.M = pc.Z = pc.W = pc.zf = 0.f;
-  pc.err = 0;
-  pc.zmax = -CUDART_INF_F;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) { pc.ty[i] = -CUDART_INF_F; pc.tb[i] = -1; }
-}
-// Merges q into pc.
-__device__ __forceinline__ void piece_merge(Piece &pc, const Piece &q) {
-  pc.err |= q.err;
-  pc.zmax = fmaxf(pc.zmax, q.zmax);
-  merge_stats_f(pc.M, pc.Z, pc.W, q.M, q.Z, q.W);
-  Top3 top;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) { top.y[i] = pc.ty[i]; top.b[i] = pc.tb[i]; }
-  if (q.tb[0] >= 0 && best_before(q.ty[0], q.tb[0], top.y[0], top.b[0])) pc.zf = q.zf;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) top3_insert(top, q.ty[i], q.tb[i]);
-#pragma unroll
-  for (int i = 0; i < 3; ++i) { pc.ty[i] = top.y[i]; pc.tb[i] = top.b[i]; }
-}
-
 // A row piece of this CTA is complete (all lanes hold the same pc): finishes the row, or, when the row is cut, publishes
 // the piece and finishes the row if the other pieces are all there.
 template <int DT, int SAMPLER>
@@ -408,19 +348,6 @@ __device__ __noinline__ void mark_unfinished(const uint32_t *live_rows) {
 // ---------------------------------------------------------------------------------------------
 // Samplers
 // ---------------------------------------------------------------------------------------------
-// Enters (y, b) in a list of three leaders (a warp's or a segment's); zf follows the first.  One lane.
-template <class L>
-__device__ __forceinline__ void lead_insert(L &ws, float y, int b, float z) {
-  if (top3_before(y, b, ws.ty[0], ws.tb[0])) {
-    ws.ty[2] = ws.ty[1]; ws.tb[2] = ws.tb[1]; ws.ty[1] = ws.ty[0]; ws.tb[1] = ws.tb[0]; ws.ty[0] = y; ws.tb[0] = b;
-    ws.zf = z;
-  } else if (top3_before(y, b, ws.ty[1], ws.tb[1])) {
-    ws.ty[2] = ws.ty[1]; ws.tb[2] = ws.tb[1]; ws.ty[1] = y; ws.tb[1] = b;
-  } else if (top3_before(y, b, ws.ty[2], ws.tb[2])) {
-    ws.ty[2] = y; ws.tb[2] = b;
-  }
-}
-
 // Enters a warp's leaders in its segment's list.  One lane; the list is locked for the few instructions this takes.  False
 // when the wait for the lock ran out.
 __device__ __noinline__ bool hand_in_leaders(int seg) {
@@ -439,7 +366,6 @@ __device__ __noinline__ bool hand_in_leaders(int seg) {
 // Sampler 0: scores one candidate per lane (lanes below `count`) in fp32 and enters those that may win in the warp's list.
 // best: encoded lower bound of the row's best score (the same in all lanes); returns it, raised.
 __device__ __noinline__ int score_candidates(const Candidate *queue, int count, int best) {
-  constexpr unsigned kAll = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const RowsParams &p = sm.p;
   WarpState &ws = sm.warp[threadIdx.x >> 5];
@@ -463,21 +389,7 @@ __device__ __noinline__ int score_candidates(const Candidate *queue, int count, 
     const uint4 fw = philox(p.round_key, (uint32_t)i >> 2, p.row_base + ws.row, p.ctr_lo, p.ctr_hi8 | 1u);
     y = score_f32(z, __frcp_rn(tau), cbyte, pick_word(fw, i & 3));
   }
-#pragma unroll 1
-  for (;;) {
-    valid = valid && y >= dec_float(best);  // else more than two slacks below a score already seen (or NaN)
-    if (!__any_sync(kAll, valid)) break;
-    const int e = valid ? enc_float(y) : INT_MIN, emax = __reduce_max_sync(kAll, e);
-    const int imin = __reduce_min_sync(kAll, valid && e == emax ? i : INT_MAX);
-    if (valid && e == emax && i == imin) {
-      lead_insert(ws, y, i, z);
-      valid = false;
-    }
-    __syncwarp();
-    const float ym = dec_float(emax);
-    const int enc = enc_float(ym - 4.f * score_slack(ym, p.slack_scale) - 2e-7f * fabsf(ym));
-    best = enc > best ? enc : best;
-  }
+  best = enter_leaders(ws, valid, y, i, z, best, p.slack_scale);
   __syncwarp();
   return best;
 }
@@ -1085,8 +997,6 @@ unsigned long long next_call_id() {
 std::atomic<long long> g_stall_tile{-1};
 std::atomic<unsigned long long> g_stall_wait_ns{0};
 
-constexpr unsigned long long kDefaultWaitNs = 2000000000ull;  // two seconds
-
 size_t pieces_bytes() { return (size_t)kMaxGrid * 2 * kPieceBytes; }
 
 // A launch that cannot give every SM as many tiles as it has warps spreads out until a CTA has this many: one tile for each of
@@ -1172,6 +1082,12 @@ void arm_stall(int64_t stall_tile, unsigned long long wait_ns) {
 
 cudaError_t launch_rows(const RowsParams &p, int64_t rows, int dtype, int sampler, void *workspace, size_t workspace_bytes,
                         cudaStream_t stream) {
+  if ((dtype != 0 && dtype != 1) || sampler < -1 || sampler > 1) return cudaErrorInvalidValue;
+  if (g_stall_tile.load() < 0) {  // (the hook stalls a tile of the streaming kernel)
+    bool taken = false;
+    const cudaError_t e = launch_rows_direct(p, rows, dtype, sampler, stream, taken);
+    if (taken || e != cudaSuccess) return e;
+  }
   if (dtype == 0) {
     if (sampler < 0) return launch_one<0, -1>(p, rows, workspace, workspace_bytes, stream);
     if (sampler == 0) return launch_one<0, 0>(p, rows, workspace, workspace_bytes, stream);

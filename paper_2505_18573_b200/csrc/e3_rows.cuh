@@ -10,6 +10,7 @@ constexpr int kGroup = 16;                   // vocabulary entries per coarse Ph
 constexpr int kLaneBytes = 128;              // bytes a thread takes from one tile
 constexpr int kTileBytes = 32 * kLaneBytes;  // 4 KiB: what a warp sums at a time
 constexpr int kMaxGrid = 1024;               // CTAs the piece workspace is sized for
+constexpr unsigned long long kDefaultWaitNs = 2000000000ull;  // limit of a wait inside a kernel: two seconds
 constexpr size_t kPieceBytes = 128;          // one partial row state in the workspace
 
 enum RowsMode : int { kModeSample = 0, kModeTargets = 1 };
@@ -61,5 +62,8 @@ void arm_stall(int64_t stall_tile, unsigned long long wait_ns);
 // workspace may be nullptr: rows are then never cut (whole rows per CTA).
 cudaError_t launch_rows(const RowsParams &p, int64_t rows, int dtype, int sampler, void *workspace, size_t workspace_bytes,
                         cudaStream_t stream);
+
+// The kernel of short calls; taken: whether the call is one (if not, nothing has been launched).
+cudaError_t launch_rows_direct(const RowsParams &p, int64_t rows, int dtype, int sampler, cudaStream_t stream, bool &taken);
 
 }  // namespace e3

@@ -486,30 +486,33 @@ __device__ __noinline__ SlowTile<DT> tile_slow(uint32_t B, int n, bool over, boo
   return s;
 }
 
+// The 16 bytes that begin `a` bytes (1..15) into the 32 bytes x, y.
+__device__ __forceinline__ uint4 shift_vec(const uint4 &x, const uint4 &y, uint32_t a) {
+  const uint32_t q = a >> 2, sh = (a & 3u) * 8u;
+  uint32_t w[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+  if (q & 2u) {
+#pragma unroll
+    for (int k = 0; k < 6; ++k) w[k] = w[k + 2];
+  }
+  if (q & 1u) {
+#pragma unroll
+    for (int k = 0; k < 5; ++k) w[k] = w[k + 1];
+  }
+  return make_uint4(__funnelshift_r(w[0], w[1], sh), __funnelshift_r(w[1], w[2], sh), __funnelshift_r(w[2], w[3], sh),
+                    __funnelshift_r(w[3], w[4], sh));
+}
+
 // A tile that begins `a` bytes (1..15) behind a 16-byte boundary was copied from that boundary on: moves it down by a
 // bytes within its slot (the 16 bytes behind the slot are in `spill`), 16 bytes per lane and step (the reads of a step lie at or
 // above its writes and below those of the next).
 __device__ __noinline__ void realign_tile(uint32_t base, uint32_t spill, uint32_t a) {
   const int lane = threadIdx.x & 31;
-  const uint32_t q = a >> 2, sh = (a & 3u) * 8u;
 #pragma unroll 1
   for (int i = 0; i < 8; ++i) {
     const uint32_t addr = base + (uint32_t)(i * 512 + lane * 16);
-    const uint4 x = lds128(addr), y = lds128(i == 7 && lane == 31 ? spill : addr + 16);
-    uint32_t w[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
-    if (q & 2u) {
-#pragma unroll
-      for (int k = 0; k < 6; ++k) w[k] = w[k + 2];
-    }
-    if (q & 1u) {
-#pragma unroll
-      for (int k = 0; k < 5; ++k) w[k] = w[k + 1];
-    }
-    uint32_t o[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) o[k] = __funnelshift_r(w[k], w[k + 1], sh);
+    const uint4 o = shift_vec(lds128(addr), lds128(i == 7 && lane == 31 ? spill : addr + 16), a);
     __syncwarp();
-    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]) : "memory");
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(o.x), "r"(o.y), "r"(o.z), "r"(o.w) : "memory");
     __syncwarp();
   }
   fence_async_smem();  // the next bulk copy into the slot comes after these stores
@@ -585,8 +588,8 @@ __device__ __noinline__ double exact_score(float zf, float tau, uint32_t cbyte, 
   return s + (-log(-log(u)));
 }
 
-// fp32 value of y_i for fine word xw, coarse byte cbyte (within score_slack of the exact value).
-__device__ __forceinline__ float score_f32(float zf, float inv_tau, uint32_t cbyte, uint32_t xw) {
+// fp32 Gumbel variate for coarse byte cbyte, fine word xw.
+__device__ __forceinline__ float gumbel_f32(uint32_t cbyte, uint32_t xw) {
   float w;  // -ln u
   if (cbyte == 255u) {
     // 1 - u = (2^32 - x - 1/2) 2^-40 < 2^-8 and -ln u = d + d^2/2 + d^3/3 + ...
@@ -596,7 +599,11 @@ __device__ __forceinline__ float score_f32(float zf, float inv_tau, uint32_t cby
     const float u = ((float)cbyte + ((float)xw + 0.5f) * 0x1p-32f) * 0.00390625f;
     w = -lg2f(u) * kLn2f;
   }
-  return fmaf(zf, inv_tau, -lg2f(w) * kLn2f);
+  return -lg2f(w) * kLn2f;
+}
+// fp32 value of y_i (within score_slack of the exact value).
+__device__ __forceinline__ float score_f32(float zf, float inv_tau, uint32_t cbyte, uint32_t xw) {
+  return fmaf(zf, inv_tau, gumbel_f32(cbyte, xw));
 }
 
 __device__ __forceinline__ bool best_before(float y, int i, float y2, int i2) {
@@ -720,6 +727,32 @@ __device__ __forceinline__ void warp_merge_top(Top3 &top, float &zf) {
       const bool mine = c2 && hb == bmin;
       if (r == 0) zf = __shfl_sync(kAll, zf, __ffs(__ballot_sync(kAll, mine)) - 1);
       if (mine) ++pos;
+    }
+  }
+  top = out;
+}
+
+// The same, but what lies further than `near` below the largest score is left out (none of it: index -1), which takes one round
+// where no two scores are that close.
+__device__ __forceinline__ void warp_merge_near(Top3 &top, float near_scale, float near_rel) {
+  constexpr unsigned kAll = 0xffffffffu;
+  Top3 out;
+  top3_reset(out);
+  float hy = top.y[0];
+  int hb = top.b[0];
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    const int e = hb >= 0 ? enc_float(hy) : INT_MIN, emax = __reduce_max_sync(kAll, e);
+    if (emax == INT_MIN) break;
+    const float y = dec_float(emax);
+    if (r > 0 && !(out.y[0] - y <= near_scale + near_rel * fabsf(out.y[0]))) break;
+    const int bmin = __reduce_min_sync(kAll, e == emax ? hb : INT_MAX);
+    out.y[r] = y;
+    out.b[r] = bmin;
+    if (e == emax && hb == bmin) {
+      hy = top.y[1]; hb = top.b[1];
+      top.y[1] = top.y[2]; top.b[1] = top.b[2];
+      top.b[2] = -1;
     }
   }
   top = out;
@@ -860,19 +893,14 @@ __device__ __noinline__ int draw_in_block_exact(const EvalCtx &x, int b, int lan
 // The same draw in fp32.  The prefix sums are good to about 3e-6 of the block sum (entries that matter
 // have |t| < 25, so the rounding of t costs 2e-6 relative, `ex2` 2e-7, the 13 additions 8e-7); when the
 // threshold comes closer than ten times that to a prefix boundary the exact form decides.
-// z_tok: logit of the token.
+// z: the lane's eight logits of the block (-inf beyond the row); word: draw_word(x); z_tok: logit of the token.
+__device__ __forceinline__ uint32_t draw_word(const EvalCtx &x) { return philox(x.rk, 0u, x.grow, x.ctr_lo, x.ctr_hi8 | 3u).x; }
 template <int DT>
-__device__ __noinline__ int draw_in_block(const EvalCtx &x, int b, int lane, float &z_tok) {
-  float z[8];
+__device__ __forceinline__ int draw_among(const EvalCtx &x, int b, int lane, const float (&z)[8], uint32_t word, float &z_tok) {
   float m = -CUDART_INF_F;
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const int i = b * 256 + lane * 8 + k;
-    z[k] = i < x.V ? load_elem<DT>(x.row, i) : -CUDART_INF_F;
-    m = fmaxf(m, z[k]);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  for (int k = 0; k < 8; ++k) m = fmaxf(m, z[k]);
+  m = dec_float(__reduce_max_sync(0xffffffffu, enc_float(m)));
   int tok = -1;
   bool exact = !(m > -CUDART_INF_F && m < CUDART_INF_F);
   if (!exact) {
@@ -892,8 +920,7 @@ __device__ __noinline__ int draw_in_block(const EvalCtx &x, int b, int lane, flo
     }
     const float total = __shfl_sync(0xffffffffu, incl, 31);
     const float before = incl - run;
-    const uint4 w3 = philox(x.rk, 0u, x.grow, x.ctr_lo, x.ctr_hi8 | 3u);
-    const float t = (float)((((double)w3.x + 0.5) * 0x1p-32) * (double)total);
+    const float t = (float)((((double)word + 0.5) * 0x1p-32) * (double)total);
     int hit = -1;
     float gap = CUDART_INF_F;
 #pragma unroll
@@ -902,8 +929,7 @@ __device__ __noinline__ int draw_in_block(const EvalCtx &x, int b, int lane, flo
       if (pk > t) hit = k;
       gap = fminf(gap, fabsf(pk - t));
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) gap = fminf(gap, __shfl_xor_sync(0xffffffffu, gap, o));
+    gap = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(gap)));  // (not negative: ordered like its bits)
     const uint32_t found = __ballot_sync(0xffffffffu, hit >= 0);
     exact = !(gap > 3e-5f * total) || found == 0u || !(total > 0.f) || !(total < CUDART_INF_F);
     if (!exact) {
@@ -923,14 +949,29 @@ __device__ __noinline__ int draw_in_block(const EvalCtx &x, int b, int lane, flo
   return tok;
 }
 
+template <int DT>
+__device__ __noinline__ int draw_in_block(const EvalCtx &x, int b, int lane, float &z_tok) {
+  float z[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int i = b * 256 + lane * 8 + k;
+    z[k] = i < x.V ? load_elem<DT>(x.row, i) : -CUDART_INF_F;
+  }
+  return draw_among<DT>(x, b, lane, z, draw_word(x), z_tok);
+}
+
+// Whether the runner-up's score is too close to the leader's for fp32 to decide.
+__device__ __forceinline__ float block_margin(const Top3 &top) { return 1e-4f + 2e-5f * fabsf(top.y[0]); }
+__device__ __forceinline__ bool blocks_too_close(const Top3 &top) { return top.y[0] - top.y[1] <= block_margin(top); }
+
 // Picks the winning block from the three fp32 leaders (exact scores where they are too close) and
 // draws the token.  Returns -1 when the row has no block with mass.
 template <int DT>
 __device__ __noinline__ int sample_in_blocks(const EvalCtx &x, const Top3 &top, int lane, float &z_tok) {
   if (top.b[0] < 0) return -1;
   int bstar = top.b[0];
-  const float margin = 1e-4f + 2e-5f * fabsf(top.y[0]);
-  if (top.b[1] >= 0 && top.y[0] - top.y[1] <= margin) {
+  const float margin = block_margin(top);
+  if (top.b[1] >= 0 && blocks_too_close(top)) {
     double ybest = -CUDART_INF;
     int bbest = -1;
     if (top.b[2] >= 0 && top.y[0] - top.y[2] <= margin) {
@@ -992,6 +1033,105 @@ __device__ __noinline__ int settle_exact(const EvalCtx &x, const Top3 &top, floa
   warp_argmax_double(ybest, ibest, zbest);
   z_tok = zbest;
   return ibest;
+}
+
+// Enters (y, b) in a list of three leaders (a warp's or a segment's); zf follows the first.  One lane.
+template <class L>
+__device__ __forceinline__ void lead_insert(L &ws, float y, int b, float z) {
+  if (top3_before(y, b, ws.ty[0], ws.tb[0])) {
+    ws.ty[2] = ws.ty[1]; ws.tb[2] = ws.tb[1]; ws.ty[1] = ws.ty[0]; ws.tb[1] = ws.tb[0]; ws.ty[0] = y; ws.tb[0] = b;
+    ws.zf = z;
+  } else if (top3_before(y, b, ws.ty[1], ws.tb[1])) {
+    ws.ty[2] = ws.ty[1]; ws.tb[2] = ws.tb[1]; ws.ty[1] = y; ws.tb[1] = b;
+  } else if (top3_before(y, b, ws.ty[2], ws.tb[2])) {
+    ws.ty[2] = y; ws.tb[2] = b;
+  }
+}
+
+// Enters the lanes' scored candidates (y, i; logit z) that may win in a list of leaders.  best: encoded lower bound of the best score
+// (the same in all lanes); returns it, raised.
+template <class L>
+__device__ __forceinline__ int enter_leaders(L &ws, bool valid, float y, int i, float z, int best, float slack_scale) {
+  constexpr unsigned kAll = 0xffffffffu;
+#pragma unroll 1
+  for (;;) {
+    valid = valid && y >= dec_float(best);  // else more than two slacks below a score already seen (or NaN)
+    if (!__any_sync(kAll, valid)) break;
+    const int e = valid ? enc_float(y) : INT_MIN, emax = __reduce_max_sync(kAll, e);
+    const int imin = __reduce_min_sync(kAll, valid && e == emax ? i : INT_MAX);
+    if (valid && e == emax && i == imin) {
+      lead_insert(ws, y, i, z);
+      valid = false;
+    }
+    __syncwarp();
+    const float ym = dec_float(emax);
+    const int enc = enc_float(ym - 4.f * score_slack(ym, slack_scale) - 2e-7f * fabsf(ym));
+    best = enc > best ? enc : best;
+  }
+  return best;
+}
+
+__device__ __forceinline__ const char *row_ptr(const RowsParams &p, uint32_t row) { return p.logits + (size_t)row * (size_t)p.row_bytes; }
+
+// ---------------------------------------------------------------------------------------------
+// Row states and results
+// ---------------------------------------------------------------------------------------------
+struct RowInfo {
+  float c;
+  bool greedy;
+};
+
+// One thread, fp64.  zt: logit of the token whose log-probability is wanted.
+__device__ __forceinline__ void finish_row(const RowsParams &p, uint32_t row, const RowInfo &ri, float Mf, float Zf,
+                                           float Wf, float zmax, int idx, int err, bool have_zt, float zt) {
+  const double M = Mf, Z = Zf, W = Wf;
+  const bool sample = p.mode == kModeSample;
+  int tok = -1;
+  float logp = CUDART_NAN_F, ent = CUDART_NAN_F, gap = CUDART_NAN_F;
+  if (ri.greedy) {
+    if (err == 0 && idx >= 0) { tok = idx; logp = 0.f; ent = 0.f; gap = 0.f; }
+  } else if (err == 0 && Z > 0.0) {
+    const double lnZ = log(Z), mean = W / Z;
+    ent = (float)(lnZ - kLn2 * mean);
+    // sum p_i (s_max - s_i) with s = z/tau: the mean of s is (M + W/Z) ln2
+    gap = (float)(((double)zmax * (double)ri.c - M - mean) * kLn2);
+    if (sample) tok = idx;
+    if (have_zt) logp = (float)(((double)zt * (double)ri.c - M) * kLn2 - lnZ);
+  }
+  if (p.out_ent) p.out_ent[row] = ent;
+  if (p.out_gap) p.out_gap[row] = gap;
+  if (sample) p.out_tok[row] = tok;
+  if (p.out_logp) p.out_logp[row] = logp;
+}
+
+// A row without a result: masked out (v = 0) or given up on because a wait ran out (v = NaN).
+__device__ __forceinline__ void write_plain(const RowsParams &p, uint32_t row, float v) {
+  if (p.mode == kModeSample) p.out_tok[row] = -1;
+  if (p.out_logp) p.out_logp[row] = v;
+  if (p.out_ent) p.out_ent[row] = v;
+  if (p.out_gap) p.out_gap[row] = v;
+}
+
+__device__ __forceinline__ void piece_reset(Piece &pc) {
+  pc.M = pc.Z = pc.W = pc.zf = 0.f;
+  pc.err = 0;
+  pc.zmax = -CUDART_INF_F;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) { pc.ty[i] = -CUDART_INF_F; pc.tb[i] = -1; }
+}
+// Merges q into pc.
+__device__ __forceinline__ void piece_merge(Piece &pc, const Piece &q) {
+  pc.err |= q.err;
+  pc.zmax = fmaxf(pc.zmax, q.zmax);
+  merge_stats_f(pc.M, pc.Z, pc.W, q.M, q.Z, q.W);
+  Top3 top;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) { top.y[i] = pc.ty[i]; top.b[i] = pc.tb[i]; }
+  if (q.tb[0] >= 0 && best_before(q.ty[0], q.tb[0], top.y[0], top.b[0])) pc.zf = q.zf;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) top3_insert(top, q.ty[i], q.tb[i]);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) { pc.ty[i] = top.y[i]; pc.tb[i] = top.b[i]; }
 }
 
 }  // namespace

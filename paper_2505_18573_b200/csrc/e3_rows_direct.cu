@@ -582,7 +582,7 @@ Plan plan(int64_t rows, int64_t V, int64_t esize, int sampler, bool mask, int64_
   auto fits = [&](int64_t ctas, int64_t bytes) { return ctas >= 1 && chunk_of(V, ctas) * esize <= bytes; };
   auto least_of = [](int64_t a, int64_t b, int64_t c) { return a < b ? (a < c ? a : c) : (b < c ? b : c); };
   int64_t ctas = least_of(most, (V + 4095) / 4096, two);
-  if (fits(ctas, 16 * 1024)) return Plan{256, (int)ctas};
+  if (fits(ctas, 12 * 1024)) return Plan{256, (int)ctas};
   ctas = least_of(most, (V + 8191) / 8192, two);
   if (fits(ctas, kChunkBytes)) return Plan{512, (int)ctas};
   const int64_t waves_percent = mask ? 400 : (sampler == 0 ? 200 : 110);

@@ -6,12 +6,16 @@
 // is bound by HBM traffic (read + write).  The row's normaliser is not recomputed: the forward pass
 // returned ln p_tok, and ln p_i = (z_i - z_tok)/tau + ln p_tok.
 //
-// Work items are (row, segment of 8,192 entries), one CTA each,
-// each thread moving 16-byte vectors (8 bf16 or 4 fp32 logits) with streaming loads and stores.  A row of an odd
-// vocabulary begins anywhere: its vectors start at the first 16-byte boundary, the few entries before it go one by one.  That
-// takes logits and gradients which lie equally far behind a boundary (the same tensor shape and layout gives that); where
-// they do not, the row goes entry by entry (300 x 33,333 fp32, 106 of the rows masked and only written: 28.1 us that way, 13.5 us
-// with vectors, 4,900 GB/s).
+// Work items are (row, segment), one CTA each, each thread moving 16-byte vectors (8 bf16 or 4 fp32 logits) with streaming loads and
+// stores: eight vectors per thread (32 KB of logits per item) where there are many items, because a CTA must have enough under way (bf16
+// with four: 2,048 x 151,936, 1,774 rows unmasked, 182 us, with eight 173), four where items are what there is too few of (128 x 45,000
+// bf16: 5.5 and 7.0 us).  What a CTA waits for before its logits is the mask alone: the row's other numbers are under way beside it, and
+// the target's logit, which needs one of them, beside the logits.  One after the other these loads cost 188 us instead of 182 on the
+// first case and 12.0 instead of 10.6 on 128 x 64,000 fp32.
+// A row of an odd vocabulary begins anywhere: its vectors start at the first 16-byte boundary, the few entries before it go one by one.
+// That takes logits and gradients which lie equally far behind a boundary (the same tensor shape and layout gives that); where
+// they do not, the row goes entry by entry (300 x 33,333 fp32, 106 of the rows masked and only written: 28.1 us that way, 12.8 us
+// with vectors, 5,100 GB/s).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math_constants.h>
@@ -22,7 +26,9 @@
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kSegE = 8192;  // entries per work item
+// Items of eight vectors per thread from which on they are taken: seven waves of four per SM (us with four and eight: 256 x 100,000 fp32,
+// 3,328 items, 28.0 and 28.6; 512 x 128,000 bf16, 4,096 items, 34.6 and 33.3; 1,024 x 128,000 fp32, 16,384 items, 127.5 and 124.3).
+constexpr int64_t kWideItems = 4096;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 
@@ -83,11 +89,13 @@ __device__ __forceinline__ void store_grad(void *base, int64_t idx, float v) {
 }
 
 template <int DT>
-__global__ void __launch_bounds__(kThreads) backward_kernel(const BwdParams p) {
+constexpr int kVectorE = DT == 0 ? 4 : 8;  // entries per 16-byte vector
+
+template <int DT, int kPerThread>
+__global__ void __launch_bounds__(kThreads, kPerThread == 8 ? 4 : 5) backward_kernel(const BwdParams p) {
   constexpr int kEsize = DT == 0 ? 4 : 2;
-  constexpr int kVecE = DT == 0 ? 4 : 8;            // entries per 16-byte vector
-  constexpr int kVecPerSeg = kSegE / kVecE;
-  constexpr int kPerThread = kVecPerSeg / kThreads;  // 8 fp32 / 4 bf16 vectors per thread and item
+  constexpr int kVecE = kVectorE<DT>;
+  constexpr int kSegE = kThreads * kPerThread * kVecE;  // entries per work item
   // programmatic dependent launch: nothing in global memory is touched before the wait, which returns once
   // the kernel before this one in the stream has completed
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -96,29 +104,27 @@ __global__ void __launch_bounds__(kThreads) backward_kernel(const BwdParams p) {
     const int64_t row = item / p.segs_per_row;
     const int e0 = (int)((item - row * p.segs_per_row) * kSegE);
     const int64_t in0 = row * p.row_stride, out0 = row * p.d_stride;
+    // Everything that depends on the row alone is asked for at once (entries of masked rows too: a few bytes), the logits as soon as the
+    // mask is known; only the target's logit waits for another load, and that beside the logits.
+    const uint8_t live = p.mask ? __ldg(p.mask + row) : 1;
+    const float tau = p.temps ? __ldg(p.temps + row) : p.temp_scalar;
+    const float lp = __ldg(p.logp + row), g_lp = p.g_logp ? __ldg(p.g_logp + row) : 0.f, g_en = p.g_ent ? __ldg(p.g_ent + row) : 0.f;
+    RowCoef k;
+    k.tok = __ldg(p.targets + row);
+    k.H = __ldg(p.ent + row);
     // 0: gradient, 1: zeros (masked row), 2: NaN (row or target not usable)
-    int kind = 0;
-    RowCoef k = {};
-    if (p.mask && __ldg(p.mask + row) == 0) {
-      kind = 1;
-    } else {
-      const float tau = p.temps ? __ldg(p.temps + row) : p.temp_scalar;
-      k.tok = __ldg(p.targets + row);
-      const float lp = __ldg(p.logp + row);
-      k.H = __ldg(p.ent + row);
-      if (!(tau > 0.f && tau < CUDART_INF_F) || k.tok < 0 || k.tok >= p.V || !(fabsf(lp) < CUDART_INF_F) ||
-          !(fabsf(k.H) < CUDART_INF_F)) {
-        kind = 2;
-      } else {
-        const float beta = 1.0f / tau;
-        k.c = __fdiv_rn(kLog2e, tau);
-        k.zt = load_logit<DT>(p.logits, in0 + k.tok);
-        k.lp2 = lp * kLog2e;
-        k.a_lp = p.g_logp ? beta * __ldg(p.g_logp + row) : 0.f;
-        k.a_en = p.g_ent ? beta * __ldg(p.g_ent + row) : 0.f;
-      }
-    }
-    const float fill = kind == 1 ? 0.f : CUDART_NAN_F;
+    auto kind_of = [&]() {
+      if (live == 0) return 1;
+      return !(tau > 0.f && tau < CUDART_INF_F) || k.tok < 0 || k.tok >= p.V || !(fabsf(lp) < CUDART_INF_F) || !(fabsf(k.H) < CUDART_INF_F) ? 2 : 0;
+    };
+    auto coefficients = [&]() {
+      const float beta = 1.0f / tau;
+      k.c = __fdiv_rn(kLog2e, tau);
+      k.zt = load_logit<DT>(p.logits, in0 + k.tok);
+      k.lp2 = lp * kLog2e;
+      k.a_lp = beta * g_lp;
+      k.a_en = beta * g_en;
+    };
     const char *const in = static_cast<const char *>(p.logits) + in0 * kEsize;
     char *const out = static_cast<char *>(p.dlogits) + out0 * kEsize;
     const int off = (int)(reinterpret_cast<uintptr_t>(in) & 15u);
@@ -133,19 +139,24 @@ __global__ void __launch_bounds__(kThreads) backward_kernel(const BwdParams p) {
       const int t = (int)threadIdx.x;
       const int lone = t < kVecE ? b0 + nvec * kVecE + t : (e0 == 0 && t - kVecE < head ? t - kVecE : (int)p.V);
       const bool alone = t < kVecE ? lone < b1 : (t < 2 * kVecE && lone < p.V);
-      if (kind != 0) {  // nothing to read: zeros or NaN
+      uint4 v[kPerThread];
+      if (live != 0) {
+#pragma unroll
+        for (int j = 0; j < kPerThread; ++j) {
+          const int vi = j * kThreads + threadIdx.x;
+          if (vi < nvec) v[j] = __ldcs(src + vi);
+        }
+      }
+      const int kind = kind_of();
+      if (kind != 0) {  // zeros or NaN
+        const float fill = kind == 1 ? 0.f : CUDART_NAN_F;
         const uint32_t f1 = DT == 0 ? __float_as_uint(fill) : (kind == 1 ? 0u : 0x7FC07FC0u);
         const uint4 o = make_uint4(f1, f1, f1, f1);
         for (int vi = threadIdx.x; vi < nvec; vi += kThreads) __stcs(dst + vi, o);
         if (alone) store_grad<DT>(p.dlogits, out0 + lone, fill);
         continue;
       }
-      uint4 v[kPerThread];
-#pragma unroll
-      for (int j = 0; j < kPerThread; ++j) {
-        const int vi = j * kThreads + threadIdx.x;
-        if (vi < nvec) v[j] = __ldcs(src + vi);
-      }
+      coefficients();
 #pragma unroll
       for (int j = 0; j < kPerThread; ++j) {
         const int vi = j * kThreads + threadIdx.x;
@@ -186,6 +197,9 @@ __global__ void __launch_bounds__(kThreads) backward_kernel(const BwdParams p) {
       if (alone) store_grad<DT>(p.dlogits, out0 + lone, grad_entry(k, load_logit<DT>(p.logits, in0 + lone), lone));
     } else {
       const int e1 = (int64_t)e0 + kSegE < p.V ? e0 + kSegE : (int)p.V;
+      const int kind = kind_of();
+      const float fill = kind == 1 ? 0.f : CUDART_NAN_F;
+      if (kind == 0) coefficients();
       for (int i = e0 + threadIdx.x; i < e1; i += kThreads)
         store_grad<DT>(p.dlogits, out0 + i, kind == 0 ? grad_entry(k, load_logit<DT>(p.logits, in0 + i), i) : fill);
     }
@@ -213,8 +227,14 @@ extern "C" e3_status e3_token_logp_entropy_backward(const void *logits, e3_dtype
   p.logits = logits; p.dlogits = dlogits; p.rows = rows; p.V = V; p.row_stride = row_stride; p.d_stride = dlogits_stride;
   p.targets = targets; p.mask = mask; p.temps = temps; p.temp_scalar = temp_scalar;
   p.logp = logp; p.ent = ent; p.g_logp = g_logp; p.g_ent = g_ent;
-  p.segs_per_row = (V + kSegE - 1) / kSegE;
-  p.items = rows * p.segs_per_row;
+  auto split = [&](int per_thread) {
+    const int64_t seg = (int64_t)kThreads * per_thread * (dt == E3_F32 ? kVectorE<0> : kVectorE<1>);
+    p.segs_per_row = (V + seg - 1) / seg;
+    p.items = rows * p.segs_per_row;
+  };
+  split(8);
+  const bool wide = p.items >= kWideItems;
+  if (!wide) split(4);
   // One CTA per item (measured faster than a grid of a few CTAs per SM that loops: the hardware hands
   // out CTAs as SMs become free, which evens out the tail); the loop only matters beyond 2^31 - 1 items.
   const int64_t cap = 0x7fffffff;
@@ -228,6 +248,7 @@ extern "C" e3_status e3_token_logp_entropy_backward(const void *logits, e3_dtype
   cfg.stream = static_cast<cudaStream_t>(stream);
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, dt == E3_F32 ? backward_kernel<0> : backward_kernel<1>, p);
+  const cudaError_t e = cudaLaunchKernelEx(
+      &cfg, dt == E3_F32 ? (wide ? backward_kernel<0, 8> : backward_kernel<0, 4>) : (wide ? backward_kernel<1, 8> : backward_kernel<1, 4>), p);
   return e == cudaSuccess ? E3_OK : E3_ERR_CUDA;
 }

@@ -135,3 +135,23 @@ def test_backward_rows_off_a_16_byte_boundary(e3, dtype, V, start):
     e3.e3_token_logp_entropy_backward(logits, targets, lp, en, g_lp, g_en, out=out)
     ref = e3.e3_token_logp_entropy_backward(logits.contiguous(), targets, lp, en, g_lp, g_en)
     assert torch.equal(out, ref) and torch.all(buf[:, :start] == 7.0) and torch.all(buf[:, start + V:] == 7.0)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("rows, V, stride", [(4100, 5001, 5001), (4100, 4096, 4104), (1400, 33333, 33333), (1400, 32768, 32768), (2100, 16385, 16392)])
+def test_backward_of_many_rows_as_of_few(e3, dtype, rows, V, stride):
+    """Items of eight vectors per thread and of four: the same bits."""
+    g = torch.Generator(device=DEV); g.manual_seed(V)
+    logits = (torch.randn((rows, stride), generator=g, device=DEV) * 3).to(dtype)[:, :V]
+    targets = inputs.uniform_targets(rows, V, seed=1, device=DEV)
+    mask = (torch.rand(rows, generator=g, device=DEV) < 0.8).to(torch.uint8)
+    temps = inputs.uniform_temps(rows, seed=2, device=DEV)
+    lp, en = e3.e3_token_logp_entropy(logits, targets, mask=mask, temps=temps)
+    g_lp, g_en = torch.randn(rows, generator=g, device=DEV), torch.randn(rows, generator=g, device=DEV)
+
+    def call(lo, hi):
+        out = torch.full((hi - lo, stride), 7.0, dtype=dtype, device=DEV)
+        e3.e3_token_logp_entropy_backward(logits[lo:hi], targets[lo:hi], lp[lo:hi], en[lo:hi], g_lp[lo:hi], g_en[lo:hi],
+                                          mask=mask[lo:hi], temps=temps[lo:hi], out=out[:, :V])
+        return out
+    assert torch.equal(call(0, rows), torch.cat([call(lo, min(lo + 300, rows)) for lo in range(0, rows, 300)]))

@@ -55,11 +55,13 @@
 // gating or on fp32.
 //
 // Sampler 1 (one Gumbel per block of 256 entries).  4 or 8 neighbouring lanes hold a block of the tile: two or three
-// shuffles add their sums up, and the block's log-sum-exp is added to its score in shared memory.  The Gumbel variates do not
-// depend on the logits: the warp that takes the first strip of a segment makes all of the segment's (four per Philox call)
-// and adds them to the scores (two addends: their order does not matter).  The segment's finisher keeps three leaders (fp32);
-// the row's finisher settles near-ties of block scores in fp64 and draws inside the winning block by inverse CDF (fp32,
-// fp64 near a prefix boundary).
+// shuffles add their sums up.  The Gumbel variates do not depend on the logits: a warp makes those of its strip (four per Philox
+// call, one call per lane) while the strip's first tile is under way, adds the blocks' log-sum-exps to them, and leaves the strip's
+// leading blocks beside its record (one, and two more only where they come close).  The segment's finisher merges those; the row's
+// finisher settles near-ties of block scores in fp64 and draws inside the winning block by inverse CDF (fp32, fp64 near a prefix
+// boundary).  With the scores of all blocks in a ring of shared memory instead (512 tiles of them, the variates of a segment made by the warp
+// that took its first strip, added up by atomics, looked through by the segment's finisher) strips could be four tiles long at most in
+// a long run: 4,096 x 151,936 bf16 235 us, now 216, 512 rows 41.2, now 38.3, 256 x 256,000 fp32 64.7, now 49.7.
 #include "e3_rows.cuh"
 #include "e3_rows_device.cuh"
 #include "e3_rows_split.cuh"
@@ -75,7 +77,7 @@ constexpr int kThreads = kWarps * 32;
 constexpr int kStages = 2;       // ring slots per warp
 constexpr int kMaxLive = 1024;   // rows of a CTA's run with a response mask (their numbers are kept in shared memory)
 constexpr int kQueueCap = 64;    // sampler 0: a push meets at most 31 entries and adds at most 32
-constexpr int kMaxBlocks = kBlockScoreTiles * 8;  // sampler 1: blocks whose scores the CTA keeps
+constexpr int kStripBlocks = kBlockStripTiles * 8;  // sampler 1: most blocks of a strip
 
 // An entry of sampler 0 that may win: vocabulary index (with kAnyByte: its coarse byte has not been looked at, else it is
 // 255) and logit.
@@ -107,7 +109,7 @@ struct WarpState {
 
 // A segment: what its warps have handed in.  At the ring place of its first strip.
 struct Segment {
-  int arrived;     // strips summed (sampler 1: + 1 for the Gumbel variates)
+  int arrived;     // strips summed
   int lock, err;
   float ty[3], zf;
   int tb[3];       // (training side: tb[0] = the target, once its logit has come by)
@@ -117,6 +119,12 @@ struct Segment {
 struct LongPiece {
   int q0, turn;    // first strip; segments merged
   Piece state;
+};
+
+// Sampler 1: the leading blocks of a strip (further ones than the first only where they come close to it; index -1: none).
+struct BlockLeaders {
+  float y[3];
+  int b[3];
 };
 
 struct Smem {
@@ -256,7 +264,7 @@ __device__ __noinline__ void finish_piece(const Piece &pc_in, int j, bool whole,
 // The warp that completes the segment whose first strip is number q merges its records, in their order, and gives their
 // places free.  With the row piece's last segment the piece is complete.  False when a wait was given up.
 template <int DT, int SAMPLER>
-__device__ __noinline__ bool finish_segment(int q, uint32_t row, float tau, float *score) {
+__device__ __noinline__ bool finish_segment(int q, uint32_t row, float tau, const BlockLeaders *blocks) {
   const RowsParams &p = sm.p;
   const int lane = threadIdx.x & 31;
   const Place w = place_of(p, sm.run, q);
@@ -276,19 +284,15 @@ __device__ __noinline__ bool finish_segment(int q, uint32_t row, float tau, floa
 #pragma unroll
   for (int i = 0; i < 3; ++i) { pc.ty[i] = sg.ty[i]; pc.tb[i] = sg.tb[i]; }
   if (SAMPLER == 1) {
-    constexpr int kBT = Fmt<DT>::kBT;
     Top3 top;
     top3_reset(top);
-    const int t0 = w.strip * p.strip_tiles, t1 = t0 + n * p.strip_tiles < p.tpr ? t0 + n * p.strip_tiles : p.tpr;
-    const int at0 = (q & mask) * p.strip_tiles * kBT, all = p.ring * p.strip_tiles * kBT;
-    for (int e = lane; e < (t1 - t0) * kBT; e += 32) {
-      const int at = at0 + e < all ? at0 + e : at0 + e - all;
-      const float y = score[at];
-      score[at] = 0.f;  // (the place's next use adds to it)
-      if (y > -CUDART_INF_F) top3_insert(top, y, t0 * kBT + e);  // a block without mass (or beyond the row) takes no part
+    for (int i = lane; i < n; i += 32) {
+      const BlockLeaders &l = blocks[(q + i) & mask];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) top3_insert(top, l.y[k], l.b[k]);
     }
-    if (tau != 0.f) {  // (greedy rows have no use for them)
-      warp_merge_top(top, pc.zf);
+    if (tau > 0.f && tau < CUDART_INF_F) {  // (the others have none)
+      merge_near_blocks(top);
 #pragma unroll
       for (int i = 0; i < 3; ++i) { pc.ty[i] = top.y[i]; pc.tb[i] = top.b[i]; }
     }
@@ -394,35 +398,57 @@ __device__ __noinline__ int score_candidates(const Candidate *queue, int count, 
   return best;
 }
 
-// Sampler 1: the Gumbel variates of the blocks of the segment that begins with strip number q, four per Philox call, added
-// to the blocks' scores.  Their places may still be in use by strips a ring's length before (earlier segments, of which this
-// warp holds no strip any more).  False when the wait for them was given up.
+// Sampler 1: the Gumbel variates of the blocks of a strip (n tiles from tile `first` of the row on), four per Philox call and lane.
 template <int DT>
-__device__ __noinline__ bool make_gumbels(int q, uint32_t row, float *score) {
+__device__ __noinline__ void make_gumbels(uint32_t row, int first, int n, float *score) {
   constexpr int kCalls = Fmt<DT>::kBT / 4;  // per tile
+  static_assert(kStripBlocks / 4 <= 32, "one call per lane");
+  const int lane = threadIdx.x & 31;
   const RowsParams &p = sm.p;
-  const Place w = place_of(p, sm.run, q);
-  const int n = segment_strips(p, w), mask = p.ring - 1;
-  bool ok = true;
-  for (int i = threadIdx.x & 31; ok && i < n; i += 32) {
-    const int &freed = sm.freed[(q + i) & mask];
-    if (volatile_int(freed) < q + i - mask) ok = bounded_wait([&] { return volatile_int(freed) >= q + i - mask; });
-  }
-  if (!__all_sync(0xffffffffu, ok)) return false;
-  __threadfence_block();
-  const PhiloxRow prow = philox_row(p.round_key, p.row_base + row, p.ctr_lo, p.ctr_hi8 | 2u);
-  const int t0 = w.strip * p.strip_tiles, t1 = t0 + n * p.strip_tiles < p.tpr ? t0 + n * p.strip_tiles : p.tpr;
-  const int at0 = (q & mask) * p.strip_tiles * kCalls, all = p.ring * p.strip_tiles * kCalls;
-#pragma unroll 1
-  for (int e = threadIdx.x & 31; e < (t1 - t0) * kCalls; e += 32) {
-    const uint4 x = philox_call(p.round_key, prow, (uint32_t)(t0 * kCalls + e));
-    float *const at = score + 4 * (at0 + e < all ? at0 + e : at0 + e - all);
-    const uint32_t w4[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) atomicAdd(at + k, gumbel_from_word(w4[k]));
+  if (lane < n * kCalls) {
+    const uint4 x = philox(p.round_key, (uint32_t)(first * kCalls + lane), p.row_base + row, p.ctr_lo, p.ctr_hi8 | 2u);
+    *reinterpret_cast<float4 *>(score + 4 * lane) =
+        make_float4(gumbel_from_word(x.x), gumbel_from_word(x.y), gumbel_from_word(x.z), gumbel_from_word(x.w));
   }
   __syncwarp();
-  return true;
+}
+// ... the leaders of the strip's n blocks, whose scores stand in `score`; b0: number of the first.
+__device__ __noinline__ void hand_in_blocks(const float *score, int n, int b0, BlockLeaders *out) {
+  constexpr unsigned kAll = 0xffffffffu;
+  constexpr int kMine = (kStripBlocks + 31) / 32;
+  const int lane = threadIdx.x & 31;
+  __syncwarp();
+  float y[kMine], m = -CUDART_INF_F;  // (-inf: a block without mass, or beyond the row)
+#pragma unroll
+  for (int k = 0; k < kMine; ++k) {
+    y[k] = lane + 32 * k < n ? score[lane + 32 * k] : -CUDART_INF_F;
+    m = fmaxf(m, y[k]);
+  }
+  const float best = dec_float(__reduce_max_sync(kAll, enc_float(m)));
+  const float near = best - near_blocks(best);
+  int close = 0, at = INT_MAX;
+#pragma unroll
+  for (int k = kMine - 1; k >= 0; --k) {
+    close += y[k] >= near ? 1 : 0;
+    if (y[k] == best) at = b0 + lane + 32 * k;
+  }
+  Top3 top;
+  top3_reset(top);
+  if (best == -CUDART_INF_F) {
+  } else if (__reduce_add_sync(kAll, close) == 1) {
+    top.y[0] = best;
+    top.b[0] = __reduce_min_sync(kAll, at);
+  } else {
+#pragma unroll 1
+    for (int i = lane; i < n; i += 32)
+      if (score[i] > -CUDART_INF_F) top3_insert(top, score[i], b0 + i);
+    merge_near_blocks(top);
+  }
+  if (lane < 3) {
+    out->y[lane] = lane == 0 ? top.y[0] : (lane == 1 ? top.y[1] : top.y[2]);
+    out->b[lane] = lane == 0 ? top.b[0] : (lane == 1 ? top.b[1] : top.b[2]);
+  }
+  __syncwarp();
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -500,7 +526,7 @@ __device__ __noinline__ void scan_mask(uint32_t *live_rows) {
 template <int SAMPLER>
 constexpr size_t dyn_smem_bytes(bool mask) {
   return (size_t)kWarps * kStages * kTileBytes + (SAMPLER == 0 ? kWarps * kQueueCap * sizeof(Candidate) + kRing * sizeof(u64) : 0) +
-         (SAMPLER == 1 ? kMaxBlocks * sizeof(float) : 0) + (mask ? (kMaxLive + kWarps) * sizeof(uint32_t) : 0);
+         (SAMPLER == 1 ? kWarps * kStripBlocks * sizeof(float) + kRing * sizeof(BlockLeaders) : 0) + (mask ? (kMaxLive + kWarps) * sizeof(uint32_t) : 0);
 }
 
 constexpr size_t kSmemMost = 232448;  // 227 KiB
@@ -517,7 +543,8 @@ __global__ void __launch_bounds__(kThreads, 1) rows_kernel(const __grid_constant
   const int warp = __shfl_sync(kAll, tid >> 5, 0);  // (known to be the same in all lanes)
   unsigned char *const extra = dyn + kWarps * kStages * kTileBytes;
   u64 *const bests = reinterpret_cast<u64 *>(extra + kWarps * kQueueCap * sizeof(Candidate));  // sampler 0
-  float *const score = reinterpret_cast<float *>(extra);                                       // sampler 1
+  float *const score = reinterpret_cast<float *>(extra) + warp * kStripBlocks;                 // sampler 1: the warp's
+  BlockLeaders *const blocks = reinterpret_cast<BlockLeaders *>(extra + kWarps * kStripBlocks * sizeof(float));
 
   if (tid < kWarps * kStages) mbar_init(&sm.full[0][0] + tid, 1);
   if (tid < kRing) {
@@ -529,8 +556,6 @@ __global__ void __launch_bounds__(kThreads, 1) rows_kernel(const __grid_constant
     if (SAMPLER == 0) bests[tid] = 0ull;
     sm.freed[tid] = tid - p.ring + 1;
   }
-  if (SAMPLER == 1)
-    for (int i = tid; i < kMaxBlocks; i += kThreads) score[i] = 0.f;
   if (tid < kLong) sm.piece[tid].q0 = -1;
   if (tid < (int)(sizeof(RowsParams) / 4)) reinterpret_cast<uint32_t *>(&sm.p)[tid] = reinterpret_cast<const uint32_t *>(&p)[tid];
   if (tid == kThreads - 32) {
@@ -669,7 +694,7 @@ __global__ void __launch_bounds__(kThreads, 1) rows_kernel(const __grid_constant
     int target = -1;            // training side
     int best = enc_neg_inf();   // sampler 0: bound of the row's best score
     int qn = 0;                 // ... candidates in the queue
-    int count = 0, err = 0;     // strips summed (sampler 1: and the Gumbel variates made)
+    int count = 0, err = 0;     // strips summed
     int seg, need;
     {
       const StripMeta &m = sm.meta[warp][strip & 1];
@@ -691,10 +716,6 @@ __global__ void __launch_bounds__(kThreads, 1) rows_kernel(const __grid_constant
         if (SAMPLER == 0) ws.prow = philox_row(p.round_key, p.row_base + row, p.ctr_lo, p.ctr_hi8 | 0u);
       }
       if (mode & kUnusable) err = kErrValue;
-      if (SAMPLER == 1 && m.q == seg) {
-        if (!make_gumbels<DT>(seg, row, score)) break;
-        ++count;
-      }
       __syncwarp();
     }
     bool more;
@@ -702,6 +723,7 @@ __global__ void __launch_bounds__(kThreads, 1) rows_kernel(const __grid_constant
       float Zs = 0.f, Ws = 0.f, nRc = CUDART_INF_F, zmax = -CUDART_INF_F;  // the strip's sums; no reference yet
       const StripMeta &meta = sm.meta[warp][strip & 1];
       const int q = meta.q, first = meta.tile, end = meta.end;
+      if (SAMPLER == 1) make_gumbels<DT>(ws.row, first, end - first, score);
       for (int tile = first; tile < end; ++tile) {
         const int slot = done % kStages;
         // a wait that was given up ends the warp's work
@@ -890,10 +912,10 @@ __global__ void __launch_bounds__(kThreads, 1) rows_kernel(const __grid_constant
               float S = Z;
 #pragma unroll
               for (int o = 1; o < F::kLB; o <<= 1) S += __shfl_xor_sync(kAll, S, o);
-              // ln of the block's sum of exp(z/tau); -inf for a block without mass
-              if (lane % F::kLB == 0)
-                atomicAdd(score + ((q & (p.ring - 1)) * p.strip_tiles + tile - first) * F::kBT + lane / F::kLB,
-                          S > 0.f ? (lg2f(S) - nRc) * kLn2f : -CUDART_INF_F);
+              if (lane % F::kLB == 0) {  // + ln of the block's sum of exp(z/tau); -inf for a block without mass
+                float &y = score[(tile - first) * F::kBT + lane / F::kLB];
+                y = S > 0.f ? y + (lg2f(S) - nRc) * kLn2f : -CUDART_INF_F;
+              }
             }
           }
         }
@@ -911,6 +933,7 @@ __global__ void __launch_bounds__(kThreads, 1) rows_kernel(const __grid_constant
         for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(kAll, x, o);
         float *const rec = reinterpret_cast<float *>(&sm.record[q & (p.ring - 1)]);
         if ((lane & 15) == 0) *reinterpret_cast<float2 *>(rec + (low ? 0 : 2)) = low ? make_float2(-nRc, x) : make_float2(x, zmax);
+        if (SAMPLER == 1 && !(mode & (kGreedy | kUnusable))) hand_in_blocks(score, (end - first) * F::kBT, first * F::kBT, blocks + (q & (p.ring - 1)));
       }
       ++count;
       ++strip;
@@ -931,14 +954,14 @@ __global__ void __launch_bounds__(kThreads, 1) rows_kernel(const __grid_constant
       if (SAMPLER >= 0 && ws.tb[0] >= 0 && !hand_in_leaders(seg)) state = 2;
       if (state == 0) {
         __threadfence_block();
-        state = atomicAdd(&sg.arrived, count) + count == need + (SAMPLER == 1 ? 1 : 0);
+        state = atomicAdd(&sg.arrived, count) + count == need;
       }
     }
     state = __shfl_sync(kAll, state, 0);
     if (state == 2) break;
     if (state == 1) {
       __threadfence_block();
-      if (!finish_segment<DT, SAMPLER>(seg, ws.row, ws.tau, score)) break;
+      if (!finish_segment<DT, SAMPLER>(seg, ws.row, ws.tau, blocks)) break;
     }
     __syncwarp();
   }

@@ -758,6 +758,10 @@ __device__ __forceinline__ void warp_merge_near(Top3 &top, float near_scale, flo
   top = out;
 }
 
+// The leaders of sampler 1: those within twice the margin below which scores are settled in fp64.
+__device__ __forceinline__ float near_blocks(float y) { return 2e-4f + 4e-5f * fabsf(y); }
+__device__ __forceinline__ void merge_near_blocks(Top3 &top) { warp_merge_near(top, 2e-4f, 4e-5f); }
+
 // Merges the sums and largest logits held by the 32 lanes of a warp; every lane ends with the result.  A lane
 // without weight (Z = 0) takes no part.  The order of all sums is fixed by lane numbers.
 __device__ __forceinline__ void warp_merge(Piece &pc) {

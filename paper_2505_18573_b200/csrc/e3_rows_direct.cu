@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) rows_direct_kernel(
   // ---- the CTA's result
   auto merge_leaders = [&]() {
     if (SAMPLER == 0) warp_merge_near(top, 4.f * p.slack_scale * 1.7e-4f, 4.f * p.slack_scale * 1e-6f);
-    if (SAMPLER == 1) warp_merge_near(top, 2e-4f, 4e-5f);
+    if (SAMPLER == 1) merge_near_blocks(top);
 #pragma unroll
     for (int i = 0; i < 3; ++i) { pc.ty[i] = top.y[i]; pc.tb[i] = top.b[i]; }
   };

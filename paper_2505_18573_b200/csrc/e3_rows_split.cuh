@@ -15,7 +15,7 @@ namespace {
 
 constexpr int kWarps = 24;           // one CTA per SM: 80 registers a thread
 constexpr int kRing = 256;           // most strips whose records the CTA keeps (RowsParams::ring of them are)
-constexpr int kBlockScoreTiles = 512;  // sampler 1: tiles whose block scores the CTA keeps
+constexpr int kBlockStripTiles = 13;  // sampler 1: most tiles of a strip
 
 // The CTA's run of strips, numbered q = 0..len-1 in hand-out order: vocabulary order, except that the strips of the last row
 // come first when that row is cut.
@@ -108,33 +108,29 @@ E3_SPLIT int long_piece_place(const Place &w) {
 // ---- host: lengths of the strips
 // Tiles per strip.  Strips of one length keep the warps of an SM in step, so that a run of a few strips per warp takes
 // whole waves: in a short run one strip per warp is all, the shortest that does it (151,936 bf16 entries a row, us for the lengths
-// below it, at it and behind it: sampler 1 256 rows 35.2, 33.7, 27.5, 27.6, 28.5, 512 rows 45.9, 40.1, 40.2; sampler 0 512 rows 6,
-// 12, 13, 15 tiles 95, 87, 86, 94).  For the statistics that pays up to 14 tiles of bf16 and 24 of fp32, which hold half as many
-// entries (against 8 tiles: 256 x 256,000 19 tiles 46.5 and 50.6, 300 x 256,000 23 tiles 51.4 and 54.7, 512 x 100,000 17 tiles 37.7
-// and 39.6, but 768 x 100,000 25 tiles 52.0 and 50.7, 400 x 256,000 32 tiles 70.7 and 68.5), and a few blocks may hold a strip more than they have warps where the
-// last strip of a row is short (448 rows 10 tiles 28.2, 11 tiles 29.7; 512 rows 12 tiles 32.6, 13 tiles 32.8; 593 rows 14 tiles
-// 34.3, 8 tiles 36.9; 1,200 x 50,257 10 tiles 38.2, 8 tiles 40.4) but not where it is long (256 x 256,000 fp32 18 tiles 51.3) or
-// where strips are short anyway (512 x 32,000 fp32 5 tiles 18.1, 6 tiles 17.3).
+// below it, at it and behind it: sampler 1 300 rows 32.0, 28.0, 28.4; sampler 0 512 rows 6, 12, 13, 15 tiles 95, 87, 86, 94).  For the
+// statistics and sampler 1 that pays up to 14 and 13 tiles of bf16 and 24 of fp32, which hold half as many entries (against 8 tiles:
+// statistics 256 x 256,000 19 tiles 46.5 and 50.6, 300 x 256,000 23 tiles 51.4 and 54.7, 512 x 100,000 17 tiles 37.7 and 39.6, but 768 x 100,000 25
+// tiles 52.0 and 50.7, 400 x 256,000 32 tiles 70.7 and 68.5; sampler 1 256 x 256,000 49.8 and 56.9, 512 x 100,000 40.5 and 48.0), and a
+// few blocks may hold a strip more than they have warps where the last strip of a row is short (statistics 448 rows 10 tiles 28.2, 11
+// tiles 29.7; 512 rows 12 tiles 32.6, 13 tiles 32.8; 593 rows 14 tiles 34.3, 8 tiles 36.9; 1,200 x 50,257 10 tiles 38.2, 8 tiles 40.4; sampler 1 512
+// rows 12 tiles 39.0, 13 tiles 40.5) but not where it is long (256 x 256,000 fp32 18 tiles 51.3) or where strips are short anyway
+// (512 x 32,000 fp32 5 tiles 18.1, 6 tiles 17.3).
 // In a long run the waves dissolve: there a strip is as long as makes its own cost small (taking it and handing in its record
 // cost a warp about as many instructions as a tile's sums; for sampler 0 the first bound and the last look at the queue cost twice
-// that: 4,096 rows 12 tiles 537, 25 tiles 494), and for sampler 1 as short as the ring of block scores asks for (4,096 rows 4,
-// 6, 8 tiles 234, 266, 244; 1,024 rows 72, 75, 68).
+// that: 4,096 rows 12 tiles 537, 25 tiles 494; sampler 1, 4,096 rows 4, 6, 8, 12 tiles 245, 230, 221, 230, 1,024 rows 72, 69, 67, 67).
 inline int strip_tiles(int64_t rows, int64_t tpr, int64_t ctas, int sampler, int tile_entries) {
   const int64_t warps = ctas * kWarps, per_warp = rows * tpr / warps;
-  const int64_t longest = sampler == 0 ? 25 : (sampler == 1 ? 13 : (tile_entries > 1024 ? 14 : 24));
+  const int64_t longest = sampler == 0 ? 25 : (tile_entries > 1024 ? (sampler == 1 ? 13 : 14) : 24);
   for (int64_t n = per_warp < 1 ? 1 : per_warp; n <= longest; ++n) {
     const int64_t spr = (tpr + n - 1) / n, last = tpr - (spr - 1) * n, more = rows * spr - warps;
-    if (more <= 0 || (sampler < 0 && n >= 8 && 2 * last <= n && more <= warps / 64)) return (int)n;
+    if (more <= 0 || (sampler != 0 && n >= 8 && 2 * last <= n && more <= warps / 64)) return (int)n;
   }
   if (sampler == 0) return 25;
-  return sampler == 1 && per_warp >= 32 ? 4 : 8;
+  return 8;
 }
-// Strips whose records a CTA keeps: sampler 1 keeps the scores of kBlockScoreTiles tiles' blocks.
-inline int ring_strips(int strip, int sampler) {
-  int ring = kRing;
-  while (sampler == 1 && ring * strip > kBlockScoreTiles) ring /= 2;
-  return ring;
-}
+// Strips whose records a CTA keeps (whatever their length and the sampler).
+inline int ring_strips(int /*strip*/, int /*sampler*/) { return kRing; }
 
 }  // namespace
 }  // namespace e3

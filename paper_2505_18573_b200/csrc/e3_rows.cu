@@ -878,12 +878,27 @@ __global__ void __launch_bounds__(kThreads, 1) rows_kernel(const __grid_constant
                   const int j = over != 0u ? __ffs((int)over) - 1 : 0;
                   const int g = e_lane + ((j ^ ga) << 4);
                   uint32_t above = 0u;  // bit k: entry k of the group
-                  {
+                  // bf16: compared in pairs as they are (us with the 16 entries taken apart and now: 512 x 151,936 84.3, 81.7, 4,096 x 9,000
+                  // 88.6, 85.1; fp32 gains nothing, 256 x 256,000 81.0, 82.0)
+                  if (DT == 1) {
+                    if (over != 0u) {
+                      float zg = Zg[0];
+#pragma unroll
+                      for (int i = 1; i < kG; ++i) zg = j == i ? Zg[i] : zg;
+                      const float top = zg > first_thr ? gate_hi : CUDART_INF_F;  // (entries above it have been looked at)
+#pragma unroll
+                      for (int i = 0; i < F::kVG; ++i) {
+                        const uint4 v = lds128(base + (uint32_t)(g * F::kEsize + 16 * i));
+                        above |= (entries_above<DT>(v, gate) & ~entries_above<DT>(v, top)) << (8 * i);
+                      }
+                      if (g + 16 > n) above &= g < n ? (1u << (n - g)) - 1u : 0u;
+                    }
+                  } else {
                     float z[16], zg = Zg[0];
 #pragma unroll
                     for (int i = 1; i < kG; ++i) zg = j == i ? Zg[i] : zg;
                     load_group_smem<DT>(base + (uint32_t)(g * F::kEsize), z);
-                    const float top = zg > first_thr ? gate_hi : CUDART_INF_F;  // (entries above it have been looked at)
+                    const float top = zg > first_thr ? gate_hi : CUDART_INF_F;
 #pragma unroll
                     for (int k = 0; k < 16; ++k) above |= (z[k] > gate && z[k] <= top ? 1u : 0u) << k;
                     if (over == 0u) above = 0u;

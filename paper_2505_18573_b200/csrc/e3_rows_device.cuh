@@ -3,6 +3,7 @@
 #pragma once
 #include "e3_rows.cuh"
 
+#include <cuda_bf16.h>
 #include <limits.h>
 #include <math_constants.h>
 #include <string.h>
@@ -368,6 +369,24 @@ __device__ __forceinline__ bool move_reference(float R, float c, float &nRc, flo
     nRc = up;
   }
   return true;
+}
+
+// Bit k: entry k of the vector is above the gate (bf16: above the gate rounded down to bf16, which is the same).
+template <int DT>
+__device__ __forceinline__ uint32_t entries_above(const uint4 &v, float gate) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+  uint32_t bits = 0u;
+  if (DT == 1) {
+    const __nv_bfloat162 g = __bfloat162bfloat162(__float2bfloat16_rd(gate));
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      bits |= __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&w[j]), g) & ((1u << (2 * j)) | (0x20000u << (2 * j)));
+    bits = (bits | bits >> 16) & 0xFFu;
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) bits |= (__uint_as_float(w[j]) > gate ? 1u : 0u) << j;
+  }
+  return bits;
 }
 
 // The vector number i (counted from 0 to 7 in vocabulary order) of a slice of which the first nlane entries are valid:

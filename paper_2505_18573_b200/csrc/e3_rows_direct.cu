@@ -18,8 +18,6 @@
 #include "e3_rows.cuh"
 #include "e3_rows_device.cuh"
 
-#include <cuda_bf16.h>
-
 #include <atomic>
 #include <mutex>
 #include <type_traits>
@@ -97,24 +95,6 @@ __device__ __forceinline__ void load_vecs(uint32_t base, uint32_t a, uint32_t of
 #pragma unroll
     for (int i = 0; i < N; ++i) v[i] = mask_vec<DT>(v[i], valid, i ^ sw);
   }
-}
-
-// Bit k: entry k of the vector is above the gate (bf16: above the gate rounded down).
-template <int DT>
-__device__ __forceinline__ uint32_t entries_above(const uint4 &v, float gate) {
-  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-  uint32_t bits = 0u;
-  if (DT == 1) {
-    const __nv_bfloat162 g = __bfloat162bfloat162(__float2bfloat16_rd(gate));
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      bits |= __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&w[j]), g) & ((1u << (2 * j)) | (0x20000u << (2 * j)));
-    bits = (bits | bits >> 16) & 0xFFu;
-  } else {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) bits |= (__uint_as_float(w[j]) > gate ? 1u : 0u) << j;
-  }
-  return bits;
 }
 
 template <int DT, int SAMPLER, int kThreads>

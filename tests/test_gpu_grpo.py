@@ -130,3 +130,20 @@ def test_advantages_are_laid_out_like_the_rewards(e3):
     assert torch.equal(turned.t(), want) and torch.equal(flags, turned_flags)
     adv, _ = e3.e3_group_advantage(torch.zeros(0, device=DEV), off[:1] * 0, out_flags=torch.zeros(0, dtype=torch.uint8, device=DEV))
     assert adv.numel() == 0
+
+
+@pytest.mark.parametrize("sizes,seq_len,min_len", [
+    ([1], 1, 1), ([16], 128, 1), ([17], 127, 0), ([2, 0, 14, 0], 33, 0), ([64, 64], 128, 0), ([64, 64], 129, 0), ([64, 65], 128, 0),
+    ([5] * 3 + [0] * 1100, 40, 0), ([40] * 20, 2049, 0)])
+def test_grpo_objective_at_the_edges_of_one_launch(e3, sizes, seq_len, min_len):
+    """Up to 128 responses of up to 128 tokens are one launch; one more response, token or many more (empty) groups are not."""
+    logp, logp_old, mask, adv, off = _case(seq_len, sizes, seq_len, min_len)
+    adv = adv + np.float32(0.3)  # (groups of one)
+    t = lambda a: torch.from_numpy(a).to(DEV)
+    for m in (mask, None):
+        out, g = e3.e3_grpo_objective(t(logp), t(logp_old), t(adv), t(off), mask=None if m is None else t(m))
+        J, grad, frac = oracle.grpo_objective(logp, logp_old, m, adv, off, 0.2)
+        assert float(out[0]) == pytest.approx(J, abs=1e-12) and float(out[1]) == pytest.approx(frac, abs=1e-12)
+        got = g.cpu().numpy().astype(np.float64)
+        assert np.array_equal(got == 0, grad == 0)
+        assert np.all(np.abs(got - grad) <= np.abs(grad) * 2.0 ** -23 + 1e-30)

@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(kShortThreads) grpo_short_kernel(const float *
     }
     part = total;
   }
-  cluster.sync();
+  if (gridDim.x > 1) cluster.sync();
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     for (unsigned r = 1; r < cluster.num_blocks(); ++r) {
       const SeqPartial *q = cluster.map_shared_rank(&part, r);
@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(kShortThreads) grpo_short_kernel(const float *
     *out_J = n_groups > 0 ? total.J / (double)n_groups : 0.0;
     if (out_clip_frac) *out_clip_frac = total.tokens > 0.0 ? total.clipped / total.tokens : 0.0;
   }
-  cluster.sync();  // the other blocks' shared memory stays until it has been read
+  if (gridDim.x > 1) cluster.sync();  // the other blocks' shared memory stays until it has been read
 }
 
 __global__ void __launch_bounds__(kThreads) grpo_final_kernel(const SeqPartial *__restrict__ part, int64_t n_seq,

@@ -554,6 +554,10 @@ cudaError_t launch(const RowsParams &p, int64_t rows, int ctas, int dev, cudaStr
 // it: 100 x 64,000 fp32 15.1 (streaming 17.1), 600 x 20,000 bf16 15.2 (16.1), but 1,000 x 20,000 21.2 (20.0).  Sampler 0 gains more here than a
 // second wave costs: 1,000 x 20,000 31.6 (48.6), 128 x 151,936 35.9 (41.7), 256 x 151,936 62.2 (57.5); and of the CTAs of a call with a
 // response mask many have nothing to do: 1,024 x 32,000, 640 of them unmasked, 17.0 (22.5).
+// Where one block takes a whole row of 32 KB or more, more waves still pay: with a mask 4,096 x 20,000 bf16, 2,560 rows unmasked, 31.7
+// (34.5), nearly all unmasked 43.8 (45.8), 2,048 x 25,000 fp32 29.3 (36.5), 2,048 x 32,000 bf16 26.4 (29.6), 2,400 x 35,000 33.6 (32.6), and all 1,500 rows
+// of 50,000 unmasked 41.5 (39.4), but 8,192 x 32,000 87.1 (71.3); sampler 0 1,500 x 32,000 63.5 (72.1), 3,000 x 32,000 116 (113); without a mask
+// the streaming kernel has no mask to count.
 struct Plan {
   int threads, ctas;
 };
@@ -570,6 +574,13 @@ Plan plan(int64_t rows, int64_t V, int64_t esize, int sampler, bool mask, int64_
     if (!fits(ctas, 70 * 1024)) continue;
     const int64_t smem = chunk_of(V, ctas) * esize + 6 * 1024, per_sm = 227 * 1024 / smem < 4 ? 227 * 1024 / smem : 4;
     if (rows * ctas * 100 <= per_sm * sms * waves_percent) return Plan{256, (int)ctas};
+  }
+  // one block a row
+  const int64_t row = chunk_of(V, 1) * esize, waves = mask ? 7 : (sampler == 0 ? 4 : 0);
+  if (row >= 32 * 1024 && row <= kChunkBytes) {
+    const int64_t threads = row <= 70 * 1024 ? 256 : 512, fit = 227 * 1024 / (row + 6 * 1024);
+    const int64_t per_sm = fit < 1024 / threads ? fit : 1024 / threads;
+    if (rows <= waves * per_sm * sms) return Plan{(int)threads, 1};
   }
   return Plan{0, 0};
 }

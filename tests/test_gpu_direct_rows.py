@@ -46,15 +46,16 @@ def _check(e3, logits, temps, mask=None):
     (3, 4095), (3, 4096), (3, 4097), (2, 65537),           # one part, two, sixteen: a last part of a few entries or of none
     (40, 16640), (40, 16641), (12, 70001),                 # parts of 256-thread blocks, of 512-thread ones; rows that begin anywhere
     (200, 26624), (200, 53248), (7, 212993), (1, 425984),  # the longest parts
-    (500, 17408), (300, 35841)])                           # three and four blocks of 256 threads per SM
+    (500, 17408), (300, 35841),                            # three and four blocks of 256 threads per SM
+    (900, 26001)])                                         # sampler 0: a block a row, more than two waves of them
 def test_parts(e3, dtype, rows, V):
     logits = inputs.zipf_gaussian_logits(rows, V, seed=rows, dtype=dtype, device=DEV)
     _check(e3, logits, inputs.uniform_temps(rows, seed=V, device=DEV))
 
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
-def test_mask(e3, dtype):
-    rows, V = 301, 20001
+@pytest.mark.parametrize("rows, V", [(301, 20001), (2000, 17001), (1300, 26100)])  # four waves, up to seven of a block a row
+def test_mask(e3, dtype, rows, V):
     logits = inputs.zipf_gaussian_logits(rows, V, seed=1, dtype=dtype, device=DEV)
     mask = (torch.rand(rows, generator=torch.Generator().manual_seed(2)) < 0.5).to(torch.uint8).to(DEV)
     logits[mask == 0] = float("nan")  # (these are not looked at)

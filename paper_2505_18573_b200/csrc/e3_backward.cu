@@ -28,6 +28,7 @@ namespace {
 constexpr int kThreads = 256;
 // Items of eight vectors per thread from which on they are taken: seven waves of four per SM (us with four and eight: 256 x 100,000 fp32,
 // 3,328 items, 28.0 and 28.6; 512 x 128,000 bf16, 4,096 items, 34.6 and 33.3; 1,024 x 128,000 fp32, 16,384 items, 127.5 and 124.3).
+// Rows for which they are not many fewer items leave threads half idle: 5,310 x 8,128 bf16 25.3 with eight, 23.4 with four.
 constexpr int64_t kWideItems = 4096;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
@@ -232,8 +233,10 @@ extern "C" e3_status e3_token_logp_entropy_backward(const void *logits, e3_dtype
     p.segs_per_row = (V + seg - 1) / seg;
     p.items = rows * p.segs_per_row;
   };
+  split(4);
+  const int64_t narrow_items = p.items;
   split(8);
-  const bool wide = p.items >= kWideItems;
+  const bool wide = p.items >= kWideItems && 5 * p.items <= 3 * narrow_items;
   if (!wide) split(4);
   // One CTA per item (measured faster than a grid of a few CTAs per SM that loops: the hardware hands
   // out CTAs as SMs become free, which evens out the tail); the loop only matters beyond 2^31 - 1 items.

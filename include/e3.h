@@ -138,7 +138,9 @@ E3_API size_t e3_workspace_bytes(e3_call which, int64_t rows, int64_t V, e3_dtyp
  *               of bytes.  For samplers other than E3_SAMPLER_BLOCK NULL (or fewer than 256 KiB) is accepted: rows are then never split, which costs
  *               throughput when there are fewer than a few thousand rows.  E3_SAMPLER_BLOCK needs the full
  *               size (E3_ERR_WORKSPACE).
- * -inf logits are allowed (probability 0, never drawn).
+ * -inf logits are allowed (probability 0, never drawn), and finite ones of any size (a fill value such as -1e9 or the type's
+ * lowest).  Where |z| / tau of a row's largest logit is above 7.4e8, fp32 has nothing between it and what has no weight beside
+ * it: logits equal to the largest share the probability.
  */
 E3_API e3_status e3_sample(const void *logits, e3_dtype dt, int64_t rows, int64_t V, int64_t row_stride,
                     const float *temps, uint64_t seed, uint64_t counter, int64_t row_base, e3_sampler sampler,

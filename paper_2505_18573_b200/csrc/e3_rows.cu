@@ -38,8 +38,9 @@
 // instruction (packed fp32).  R is the largest of a sample of 256 (bf16) or 128 (fp32) of the first tile's entries plus a
 // margin; one vote per tile checks its sums, and when an entry is far above R (or there is a NaN or a +inf) R moves up to
 // the tile's largest logit and the tile is summed again; where there is a -inf it is summed with clamped entries, and if neither
-// helps in a careful form that flags NaN and +inf.  R therefore stays close to the largest logit of the strip, which keeps W/Z small and the
-// entropy free of cancellation.  Records merge associatively; the per-row result is formed in fp64:
+// helps in a careful form that flags NaN and +inf.  R c is rounded down, so that t <= 0 up to R however large it is (a strip may begin
+// with a fill value such as -1e9); from |R c| = 2^30 on the careful form counts the entries that equal R.  R therefore stays
+// close to the largest logit of the strip, which keeps W/Z small and the entropy free of cancellation.  Records merge associatively; the per-row result is formed in fp64:
 // H = ln Z - ln2 * W / Z,  ln p_tok = (z_tok*c - M) ln2 - ln Z, and, where the caller asks for it, the mean logit gap
 // beta sum p_i Delta_i = (z_max*c - M - W/Z) ln2 of App. A.
 //
@@ -671,7 +672,6 @@ __global__ void __launch_bounds__(kThreads, 1) rows_kernel(const __grid_constant
     }
   };
 
-  enum : uint32_t { kGreedy = 1u, kUnusable = 2u, kClamped = 4u };
   bool given_up = false;
   int strip = 0;  // strips summed
   // The warp's first strip is found before the kernel waits for the one before it in the stream (8 x 32,000 bf16: 9.0 us a
@@ -789,8 +789,11 @@ __global__ void __launch_bounds__(kThreads, 1) rows_kernel(const __grid_constant
               Zs = s.Zs; Ws = s.Ws; nRc = s.nRc;
               Z = s.Z; W = s.W;
               zmax = fmaxf(zmax, s.zmax);
-              if (kLean && s.bad) err = kErrValue;
-              if (!kLean) summed = !s.bad;
+              if (kLean) {
+                err |= s.flags & kErrValue;
+                mode |= (uint32_t)s.flags & kClamped;
+              }
+              if (!kLean) summed = s.flags == 0;
               if (SAMPLER == 0) {
 #pragma unroll
                 for (int j = 0; j < kG; ++j) Zg[j] = s.Zg[j];

@@ -28,8 +28,17 @@ constexpr float kGumbelCapAll = 28.4192f;
 constexpr float kMargin = 5.f;
 constexpr float kSoundZ = 128.f;
 constexpr float kSoundW = 1e30f;  // |sum 2^t t| of a sound tile stays far below (a -inf logit makes it NaN)
+// From this size of R c on (a fill value such as -1e9 with nothing else beside it) the reference is "far": fp32 logits that differ lie 64
+// or more apart in log2 units and the rounding of R c is as large, so the sum is the number of entries that equal R.
+constexpr float kFar = 0x1p30f;
+constexpr float kFarMost = 0x1p103f;  // references are kept below this: their distance times a sum is finite
+constexpr float kClampAt = -0x1p60f;  // smaller logits enter the clamped sums as this: its product with c is finite from tau = 1e-20 on
+constexpr float kFloatMost = 3.402823466e38f;
 
 enum : int { kErrValue = 1 };
+// What a warp of the streaming kernel knows of the rows' strips in hand.  kClamped: full tiles do not take the plain sums (an entry of -inf
+// was seen, or the reference is far).
+enum : uint32_t { kGreedy = 1u, kUnusable = 2u, kClamped = 4u };
 
 template <int DT>
 struct Fmt {
@@ -276,8 +285,8 @@ __device__ __forceinline__ float warp_max(float lane_max) {
   return dec_float(__reduce_max_sync(0xffffffffu, enc_float(lane_max)));
 }
 
-// Adds the packed sums of 2^t and of 2^t t over the entries of one 16-byte vector, t = z c + nRc.  CLAMP: logits below -2^100
-// (also -inf) enter as -2^100, which gives them weight 0 and keeps 2^t t finite; NaN stays NaN.
+// Adds the packed sums of 2^t and of 2^t t over the entries of one 16-byte vector, t = z c + nRc.  CLAMP: logits below -2^60
+// (also -inf) enter as -2^60, which gives them weight 0 and keeps 2^t t finite; NaN stays NaN.
 template <int DT, bool CLAMP>
 __device__ __forceinline__ void vec_sums(const uint4 &v, f2 c2, f2 nRc2, f2 &Za, f2 &Zb, f2 &Wa, f2 &Wb) {
   const uint32_t w[4] = {v.x, v.y, v.z, v.w};
@@ -286,13 +295,13 @@ __device__ __forceinline__ void vec_sums(const uint4 &v, f2 c2, f2 nRc2, f2 &Za,
     f2 z2;
     if (DT == 1) {
       uint32_t x = w[j];
-      if (CLAMP) asm("max.NaN.bf16x2 %0, %1, %2;" : "=r"(x) : "r"(x), "r"(0xF180F180u));
+      if (CLAMP) asm("max.NaN.bf16x2 %0, %1, %2;" : "=r"(x) : "r"(x), "r"(0xDD80DD80u));
       z2 = pack2f(__uint_as_float(x << 16), __uint_as_float(x & 0xFFFF0000u));
     } else {
       float a = __uint_as_float(w[2 * j]), b = __uint_as_float(w[2 * j + 1]);
       if (CLAMP) {
-        asm("max.NaN.f32 %0, %1, %2;" : "=f"(a) : "f"(a), "f"(-1.2676506e30f));
-        asm("max.NaN.f32 %0, %1, %2;" : "=f"(b) : "f"(b), "f"(-1.2676506e30f));
+        asm("max.NaN.f32 %0, %1, %2;" : "=f"(a) : "f"(a), "f"(kClampAt));
+        asm("max.NaN.f32 %0, %1, %2;" : "=f"(b) : "f"(b), "f"(kClampAt));
       }
       z2 = pack2f(a, b);
     }
@@ -351,23 +360,54 @@ __device__ __forceinline__ float slice_max(uint32_t B) {
   return m;
 }
 
-// -R c for a strip's reference R from a sample, the lanes' first vectors; +inf: none (no finite entry there).
+// -R c, rounded down: no entry up to R has t above 0, however large R c is (rounded to nearest, a group of entries of -1e9 had t up to
+// +32, and sums beyond any limit).
+__device__ __forceinline__ float reference(float R, float c) {
+  return fminf(fmaxf(__fmul_rd(-R, c), -kFarMost), kFarMost);
+}
+// t = z c + n for entries beside a largest logit R whose R c is far: 0 for R, -64 and less for the others (both products are exact,
+// and those of clamped entries finite).  An R below the clamp becomes the clamp, as its entries do.
+__device__ __forceinline__ void far_terms(float R, float &c, float &n) {
+  R = fmaxf(R, kClampAt);
+  const int k = 31 + 127 - (int)((__float_as_uint(R) >> 23) & 255u);
+  c = __uint_as_float((uint32_t)((k < 66 ? k : 66) + 127) << 23);
+  n = -R * c;
+}
+// Entries that equal R among the `valid` first ones from `addr` on (at most 16); NaN where there is a NaN or a +inf.
+template <int DT>
+__device__ __forceinline__ float far_count(uint32_t addr, int valid, float R) {
+  float n = 0.f;
+#pragma unroll 1
+  for (int e = 0; e < kGroup && e < valid; ++e) {
+    const float z = lds_elem<DT>(addr + (uint32_t)(e * Fmt<DT>::kEsize));
+    n += z == R ? 1.f : 0.f;
+    if (!(z < CUDART_INF_F)) n = CUDART_NAN_F;
+  }
+  return n;
+}
+
+// -R c for a strip's reference R from a sample, the lanes' first vectors; +inf: none (no finite entry there, or one that is far).
 template <int DT>
 __device__ __forceinline__ float sample_reference(uint32_t B, float c) {
   const uint4 v[1] = {lds128(B)};
-  const float up = -warp_max(vec_max<DT>(v)) * c - kMargin;
-  return fabsf(up) < CUDART_INF_F ? up : CUDART_INF_F;
+  const float up = __fmaf_rd(-warp_max(vec_max<DT>(v)), c, -kMargin);
+  return fabsf(up) < kFar ? up : CUDART_INF_F;
 }
-// Moves a strip's reference up (nRc down) to the logit R and rescales its sums; false when R c leaves the fp32 range.
-__device__ __forceinline__ bool move_reference(float R, float c, float &nRc, float &Zs, float &Ws) {
-  const float up = -R * c;
-  if (!(fabsf(up) < CUDART_INF_F)) return false;
+// Moves a strip's reference down to `up`, if it lies above, and rescales its sums.
+__device__ __forceinline__ void lower_reference(float up, float &nRc, float &Zs, float &Ws) {
   if (up < nRc) {
     const float d = up - nRc, f = nRc == CUDART_INF_F ? 0.f : ex2f(d);
     Ws = f == 0.f ? 0.f : f * fmaf(d, Zs, Ws);
     Zs = f == 0.f ? 0.f : f * Zs;
     nRc = up;
   }
+}
+__device__ __forceinline__ bool is_far(float nRc) { return fabsf(nRc) >= kFar && nRc < CUDART_INF_F; }
+// The same for the logit R; false (nothing done) when there is none or R c is far.
+__device__ __forceinline__ bool move_reference(float R, float c, float &nRc, float &Zs, float &Ws) {
+  const float up = __fmul_rd(-R, c);
+  if (!(fabsf(up) < kFar)) return false;
+  lower_reference(up, nRc, Zs, Ws);
   return true;
 }
 
@@ -406,9 +446,9 @@ __device__ __forceinline__ uint4 mask_vec(const uint4 &v, int nlane, int i) {
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// The careful form, for a tile that lies only partly inside the row and for one whose sums stay out of range clamped and with its
-// largest logit as reference (a NaN, a +inf): entries are masked and clamped.  One vector per step, so that the code that few
-// tiles run stays short.
+// The careful form, for a tile that lies only partly inside the row, for one whose sums stay out of range clamped and with its
+// largest logit as reference (a NaN, a +inf), and for one whose reference is far: entries are masked and clamped.  One vector per
+// step, so that the code that few tiles run stays short.
 template <int DT>
 __device__ __forceinline__ float slice_max_careful(uint32_t B, int nlane, int r8) {
   float m = -CUDART_INF_F;
@@ -439,6 +479,22 @@ __device__ __forceinline__ void slice_sums_careful(uint32_t B, int nlane, int r8
   W = sum2(add2(Wa, Wb));
 }
 
+// The lane's groups of a tile whose reference is far: how many of their entries equal R.
+template <int DT>
+struct FarTile {
+  float Zg[Fmt<DT>::kG];
+};
+template <int DT>
+__device__ __noinline__ FarTile<DT> far_tile(uint32_t B, int nlane, float R) {
+  FarTile<DT> f;
+#pragma unroll
+  for (int j = 0; j < Fmt<DT>::kG; ++j) {
+    const int g = j ^ ((int)(threadIdx.x & 7) / Fmt<DT>::kVG);
+    f.Zg[j] = far_count<DT>((B & ~(uint32_t)(kLaneBytes - 1)) + (uint32_t)(g * kGroup * Fmt<DT>::kEsize), nlane - g * kGroup, R);
+  }
+  return f;
+}
+
 // Sums of a tile in the careful form; the strip's reference moves up to the tile's largest logit first (zmax takes it in).  True: a
 // NaN, a +inf, or numbers outside the fp32 range (the sums are 0 then).
 template <int DT>
@@ -447,10 +503,22 @@ __device__ __forceinline__ bool careful_tile(uint32_t B, int n, float c, float &
   const int lane = threadIdx.x & 31, nlane = n - lane * Fmt<DT>::kLaneE;  // entries from the lane's first on (may be < 0)
   const float R = warp_max(slice_max_careful<DT>(B, nlane, lane & 7));
   zmax = fmaxf(zmax, R);
-  bool bad = R > -CUDART_INF_F && !move_reference(R, c, nRc, Zs, Ws);
+  const float up = reference(R, c);
+  bool bad = !(c < CUDART_INF_F);
+  if (R > -CUDART_INF_F && !bad) lower_reference(up, nRc, Zs, Ws);
   // without any reference (nothing finite so far) the sums must come out as zero
   const bool none = nRc == CUDART_INF_F;
-  slice_sums_careful<DT>(B, nlane, lane & 7, c, none ? 0.f : nRc, Z, W, Zg);
+  if (is_far(nRc)) {  // (a tile below the reference counts nothing)
+    const FarTile<DT> f = far_tile<DT>(B, nlane, up == nRc ? R : CUDART_INF_F);
+    Z = W = 0.f;
+#pragma unroll
+    for (int j = 0; j < Fmt<DT>::kG; ++j) {
+      Zg[j] = f.Zg[j];
+      Z += Zg[j];
+    }
+  } else {
+    slice_sums_careful<DT>(B, nlane, lane & 7, c, none ? 0.f : nRc, Z, W, Zg);
+  }
   bad |= !(Z <= kSoundZ) || !(fabsf(W) <= kSoundW) || (none && Z != 0.f);
   bad = __any_sync(0xffffffffu, bad);
   if (bad) {
@@ -474,14 +542,14 @@ struct SlowTile {
   float Zs, Ws, nRc;  // the strip's sums and reference, moved
   float Z, W, zmax;
   float Zg[Fmt<DT>::kG];
-  bool bad;           // not summed: a NaN, a +inf, or numbers outside the fp32 range
+  int flags;          // kErrValue: not summed (a NaN, a +inf, or numbers outside the fp32 range); kClamped: see there
 };
 template <int DT, bool GROUPS, bool CAREFUL>
 __device__ __noinline__ SlowTile<DT> tile_slow(uint32_t B, int n, bool over, bool want_max, float c, float nRc, float Zs, float Ws) {
   SlowTile<DT> s;
   s.zmax = -CUDART_INF_F;
-  s.bad = true;
-  if (!CAREFUL || n == Fmt<DT>::kTileE) {
+  bool bad = true;
+  if ((!CAREFUL || n == Fmt<DT>::kTileE) && !is_far(nRc)) {
     if (nRc == CUDART_INF_F && !over) nRc = sample_reference<DT>(B, c);
     bool moved = over || nRc == CUDART_INF_F;
 #pragma unroll 1
@@ -494,14 +562,15 @@ __device__ __noinline__ SlowTile<DT> tile_slow(uint32_t B, int n, bool over, boo
       }
       if (GROUPS) slice_sums_groups<DT, true>(B, c, none ? 0.f : nRc, s.Z, s.W, s.Zg);
       else slice_sums<DT, true>(B, c, none ? 0.f : nRc, s.Z, s.W);
-      s.bad = __any_sync(0xffffffffu, !(s.Z <= (none ? 0.f : kSoundZ)) || !(fabsf(s.W) <= kSoundW));
-      if (!s.bad || moved) break;
+      bad = __any_sync(0xffffffffu, !(s.Z <= (none ? 0.f : kSoundZ)) || !(fabsf(s.W) <= kSoundW));
+      if (!bad || moved) break;
       moved = true;
     }
-    if (!s.bad && want_max) s.zmax = warp_max(slice_max<DT>(B));
+    if (!bad && want_max) s.zmax = warp_max(slice_max<DT>(B));
   }
-  if (CAREFUL && s.bad) s.bad = careful_tile<DT>(B, n, c, nRc, Zs, Ws, s.Z, s.W, s.Zg, s.zmax);
+  if (CAREFUL && bad) bad = careful_tile<DT>(B, n, c, nRc, Zs, Ws, s.Z, s.W, s.Zg, s.zmax);
   s.Zs = Zs; s.Ws = Ws; s.nRc = nRc;
+  s.flags = (bad ? kErrValue : 0) | (is_far(nRc) ? (int)kClamped : 0);
   return s;
 }
 
@@ -620,9 +689,12 @@ __device__ __forceinline__ float gumbel_f32(uint32_t cbyte, uint32_t xw) {
   }
   return -lg2f(w) * kLn2f;
 }
-// fp32 value of y_i (within score_slack of the exact value).
+// fp32 value of y_i (within score_slack of the exact value; finite for every finite logit).
+__device__ __forceinline__ float score_of(float zf, float inv_tau, float gumbel) {
+  return fminf(fmaxf(fmaf(zf, inv_tau, gumbel), -kFloatMost), kFloatMost);
+}
 __device__ __forceinline__ float score_f32(float zf, float inv_tau, uint32_t cbyte, uint32_t xw) {
-  return fmaf(zf, inv_tau, gumbel_f32(cbyte, xw));
+  return score_of(zf, inv_tau, gumbel_f32(cbyte, xw));
 }
 
 __device__ __forceinline__ bool best_before(float y, int i, float y2, int i2) {
@@ -1104,9 +1176,21 @@ struct RowInfo {
   bool greedy;
 };
 
+// A row whose reference is far: Z entries share the probability, those whose product with c rounds to the reference.
+__device__ __noinline__ void finish_far_row(const RowsParams &p, uint32_t row, float c, float M, float Z, float zmax, int idx, bool have_zt,
+                                            float zt) {
+  const double lnZ = log((double)Z);
+  auto above = [&](float z) { return -reference(z, c) == M ? 0.0 : ((double)z * (double)c - (double)M) * kLn2; };
+  if (p.out_ent) p.out_ent[row] = (float)lnZ;
+  if (p.out_gap) p.out_gap[row] = (float)above(zmax);
+  if (p.mode == kModeSample) p.out_tok[row] = idx;
+  if (p.out_logp) p.out_logp[row] = have_zt ? (float)(above(zt) - lnZ) : CUDART_NAN_F;
+}
+
 // One thread, fp64.  zt: logit of the token whose log-probability is wanted.
 __device__ __forceinline__ void finish_row(const RowsParams &p, uint32_t row, const RowInfo &ri, float Mf, float Zf,
                                            float Wf, float zmax, int idx, int err, bool have_zt, float zt) {
+  if (fabsf(Mf) >= kFar && err == 0) return finish_far_row(p, row, ri.c, Mf, Zf, zmax, idx, have_zt, zt);
   const double M = Mf, Z = Zf, W = Wf;
   const bool sample = p.mode == kModeSample;
   int tok = -1;

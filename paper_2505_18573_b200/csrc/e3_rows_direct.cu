@@ -7,6 +7,8 @@
 // coarse stream) per lane, so that 32 lanes hold two of sampler 1's blocks.  Meanwhile it makes its random numbers, which do not depend on
 // the logits: sampler 0's coarse bytes and the Gumbel variates of the entries whose byte is 255 (one in 256), sampler 1's Gumbel variates
 // and the draw inside the block.  Sums refer to the warp's largest logit so far; clamped entries (-inf) cost one instruction a pair here.
+// A warp whose 512 entries of a step are all a fill value such as -1e9 has that as its largest: its products are rounded down and,
+// where they are too large for that, taken with a power of two in place of c (far_terms), at no cost to the sums of other rows.
 // Sampler 0 scores its hits, takes the best of the CTA as bound, and scores the few entries above the gate that this leaves, whatever
 // their coarse byte.  Sampler 1 draws inside the leading block of every part, of which the row's is one.
 // The first warp merges the CTA's warps and hands the result to the first CTA of the row by `st.async` (data and signal in one); there the
@@ -95,6 +97,15 @@ __device__ __forceinline__ void load_vecs(uint32_t base, uint32_t a, uint32_t of
 #pragma unroll
     for (int i = 0; i < N; ++i) v[i] = mask_vec<DT>(v[i], valid, i ^ sw);
   }
+}
+
+// The lane's entries that equal R: groups of 16, a step of `step_e` entries apart, of which `left` entries are valid from the first on.
+template <int DT>
+__device__ __noinline__ float far_entries(uint32_t addr, int step_e, int left, float R) {
+  float n = 0.f;
+#pragma unroll 1
+  for (; left > 0; left -= step_e, addr += (uint32_t)(step_e * Fmt<DT>::kEsize)) n += far_count<DT>(addr, left, R);
+  return n;
 }
 
 template <int DT, int SAMPLER, int kThreads>
@@ -263,8 +274,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) rows_direct_kernel(
     if (__any_sync(kAll, bad)) pc.err = kErrValue;
   } else if (usable) {
     // ---- sums, relative to the largest logit of the warp so far
-    const f2 c2 = pack2f(c, c);
-    f2 nRc2 = pack2f(0.f, 0.f), Zt = nRc2, Wa = Zt, Wb = Zt;
+    f2 c2 = pack2f(c, c), nRc2 = pack2f(0.f, 0.f), Zt = nRc2, Wa = Zt, Wb = Zt;  // t = z c2 + nRc2
     float R = -CUDART_INF_F, nRc = 0.f;
 #pragma unroll 1
     for (int k = 0; k < steps; ++k) {
@@ -279,7 +289,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) rows_direct_kernel(
       }
       m = warp_max(m);
       if (m > R) {
-        const float up = -m * c;
+        const float up = reference(m, c);
         if (R > -CUDART_INF_F) {
           const float d = up - nRc, f = ex2f(d);
           Wa = fma2(pack2f(d, d), Zt, add2(Wa, Wb));
@@ -289,7 +299,10 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) rows_direct_kernel(
         }
         R = m;
         nRc = up;
-        nRc2 = pack2f(nRc, nRc);
+        float ct = c, nt = up;
+        if (fabsf(up) >= kFar) far_terms(m, ct, nt);
+        c2 = pack2f(ct, ct);
+        nRc2 = pack2f(nt, nt);
       }
       f2 Za = pack2f(0.f, 0.f), Zb = Za;
       if (valid > 0) {
@@ -308,7 +321,9 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) rows_direct_kernel(
     }
     pc.Z = sum2(Zt);
     pc.W = sum2(add2(Wa, Wb));
-    bool bad = !(pc.Z <= 1e6f) || !(fabsf(pc.W) <= kSoundW) || !(fabsf(nRc) < CUDART_INF_F);
+    if (R < kClampAt && R > -CUDART_INF_F)  // (entries of -inf are not to count)
+      pc.Z = fabsf(nRc) >= kFar ? far_entries<DT>(base + a + (uint32_t)(g0 * kGroup * F::kEsize), kStepE, n - g0 * kGroup, R) : CUDART_NAN_F;
+    bool bad = !(pc.Z <= 1e6f) || !(fabsf(pc.W) <= kSoundW) || !(c < CUDART_INF_F);
     if (R == -CUDART_INF_F) bad |= pc.Z != 0.f;
     if (__any_sync(kAll, bad)) {
       pc.err = kErrValue;
@@ -337,7 +352,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) rows_direct_kernel(
       for (;;) {
         if (hit_i >= 0) {
           const float z = lds_elem<DT>(base + a + (uint32_t)(hit_i * F::kEsize));
-          if (z > -CUDART_INF_F && z < CUDART_INF_F) top3_insert(top, fmaf(z, inv_tau, hit_g), e0 + hit_i);
+          if (z > -CUDART_INF_F && z < CUDART_INF_F) top3_insert(top, score_of(z, inv_tau, hit_g), e0 + hit_i);
         }
         if (pair < 0 && qn == 0) break;
         next_hits();

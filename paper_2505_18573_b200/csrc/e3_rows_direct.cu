@@ -406,6 +406,8 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) rows_direct_kernel(
         if (qn > 0) drain();
       }
     }
+  } else {
+    cp_async_wait(0);  // (a temperature that cannot be used: the copies still land before the CTA's memory goes to another)
   }
 
   // ---- the CTA's result

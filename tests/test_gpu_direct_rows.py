@@ -146,3 +146,25 @@ def test_graph_replay_on_cut_rows_of_the_streaming_kernel(e3, sampler):
         graph.replay()
         torch.cuda.synchronize()
         assert all(torch.equal(a, b) for a, b in zip(out, run()))
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_temperatures_that_cannot_be_used_between_others(e3, dtype):
+    """Several waves of blocks of which every other one has nothing to sum: its copies land before its memory goes to the next one."""
+    rows, V = 1100, 20001 if dtype == torch.float32 else 40001
+    logits = inputs.zipf_gaussian_logits(rows, V, seed=2, dtype=dtype, device=DEV)
+    temps = inputs.uniform_temps(rows, seed=3, device=DEV)
+    for k, bad in enumerate((-1.0, float("nan"), float("inf"))):
+        temps[2 * k::6] = bad
+    z, t = inputs.to_oracle_array(logits), temps.cpu().numpy()
+    ref = oracle.sample(z, t, 3, 4, 0, 0)
+    targets = inputs.uniform_targets(rows, V, seed=3, device=DEV)
+    mask = torch.ones(rows, dtype=torch.uint8, device=DEV)
+    rlp, ren, _ = oracle.token_logp_entropy(z, targets.cpu().numpy(), temps=t)
+    for _ in range(5):
+        tok, lp, en = e3.e3_sample(logits, temps, 3, 4)
+        assert_tokens("tok", tok.cpu().numpy(), ref)
+        assert_close("ent", en.cpu().numpy(), ref.ent, ATOL[dtype])
+        lp, en = e3.e3_token_logp_entropy(logits, targets, mask=mask, temps=temps)
+        assert_close("train.logp", lp.cpu().numpy(), rlp, ATOL[dtype])
+        assert_close("train.ent", en.cpu().numpy(), ren, ATOL[dtype])

@@ -73,6 +73,16 @@ __device__ __forceinline__ void cp_async_wait(int later) {
     default: asm volatile("cp.async.wait_group 8;" ::: "memory"); break;
   }
 }
+// One poll of a barrier that counts what other CTAs of the cluster send (their stores are visible once it says so).
+__device__ __forceinline__ bool mbar_try_wait_cluster(u64 *b, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_addr(b)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
@@ -480,11 +490,11 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) rows_direct_kernel(
     }
     if (rank != 0) return;
     __syncwarp();
-    bool came = mbar_try_wait(&sh.handed, 0);
+    bool came = mbar_try_wait_cluster(&sh.handed, 0);
     if (!__all_sync(kAll, came)) {
       const u64 t0 = global_ns();
       for (uint32_t it = 1; !came; ++it) {
-        came = mbar_try_wait(&sh.handed, 0);
+        came = mbar_try_wait_cluster(&sh.handed, 0);
         if ((it & 63u) == 0u && global_ns() - t0 > p.wait_ns) break;
       }
       if (!__all_sync(kAll, came)) {

@@ -387,6 +387,14 @@ E3_API double e3_anneal_target(const e3_sched *s);
 E3_API void e3_test_arm_stall(int64_t tile, uint64_t wait_ns);
 
 /*
+ * For tests: which kernel a row call of this size takes on a device of `sms` SMs that holds clusters of up to `largest_cluster`
+ * blocks.  0: the streaming kernel; else the kernel of short calls, with that many blocks per row.  sampler: an e3_sampler, or -1 for
+ * e3_token_logp_entropy; masked: whether that call has a mask.  No device call is made.
+ */
+E3_API int32_t e3_test_row_blocks(e3_dtype dt, int64_t rows, int64_t V, int32_t sampler, int32_t masked, int32_t sms,
+                                  int32_t largest_cluster);
+
+/*
  * Measurement aid: reads `bytes` (a multiple of 16) of device memory at `buf` (16-byte aligned) once, with a
  * plain grid of four thread blocks per SM that only adds the words up -- the practical read-only ceiling
  * of the device, against which the benchmark reports the row kernels.  `scratch`: device memory of at least

@@ -28,7 +28,7 @@ EXPORTS = ("e3_status_string", "e3_workspace_bytes", "e3_sample", "e3_token_logp
            "e3_token_logp_entropy_backward", "e3_grpo_objective",
            "e3_masked_mean_entropy", "e3_masked_mean_entropy_static", "e3_group_advantage", "e3_allocate_budget", "e3_update_temperature",
            "e3_anneal_target", "e3_entropy_gap", "e3_update_temperature_gap", "e3_difficulty_accumulate", "e3_difficulty_rank", "e3_budget_curriculum",
-           "e3_test_arm_stall", "e3_probe_read", "e3_sequence_mean_entropy")
+           "e3_test_arm_stall", "e3_test_row_blocks", "e3_probe_read", "e3_sequence_mean_entropy")
 
 
 class E3Error(RuntimeError):
@@ -116,6 +116,8 @@ def lib() -> C.CDLL:
         L.e3_anneal_target.argtypes = [C.POINTER(e3_sched)]
         L.e3_probe_read.restype = C.c_int
         L.e3_probe_read.argtypes = [C.c_void_p, C.c_size_t, C.c_void_p, C.c_size_t, C.c_void_p]
+        L.e3_test_row_blocks.restype = C.c_int32
+        L.e3_test_row_blocks.argtypes = [C.c_int, C.c_int64, C.c_int64, C.c_int32, C.c_int32, C.c_int32, C.c_int32]
         L.e3_test_arm_stall.restype = None
         L.e3_test_arm_stall.argtypes = [C.c_int64, C.c_uint64]
         _lib, _nat = L, _native
@@ -287,6 +289,11 @@ def e3_budget_curriculum(G: int, step: int, G_min_limit: int, G_max_limit: int, 
     _check("e3_budget_curriculum", st)
     return lo.value, hi.value
 
+
+
+def e3_test_row_blocks(dt: int, rows: int, V: int, sampler: int = -1, masked: bool = False, sms: int = 148, largest_cluster: int = 16) -> int:
+    """For tests: blocks per row of the kernel of short calls for a call of this size, 0 where it takes the streaming kernel."""
+    return lib().e3_test_row_blocks(dt, rows, V, sampler, int(masked), sms, largest_cluster)
 
 
 def e3_test_arm_stall(tile: int, wait_ns: int) -> None:

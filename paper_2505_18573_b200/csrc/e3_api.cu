@@ -177,4 +177,8 @@ e3_status e3::group_advantage_filled(const float *rewards, int64_t n_rewards, co
   return group_advantage(rewards, group_offsets, n_groups, eps, unbiased, out_adv, out_group_flags, n_rewards, stream);
 }
 
+extern "C" int32_t e3_test_row_blocks(e3_dtype dt, int64_t rows, int64_t V, int32_t sampler, int32_t masked, int32_t sms, int32_t largest_cluster) {
+  if ((dt != E3_F32 && dt != E3_BF16) || rows < 1 || V < 1 || V >= (int64_t(1) << 31) || sms < 1) return 0;
+  return e3::direct_ctas(rows, V, static_cast<int>(dt), sampler < 0 ? -1 : (sampler == E3_SAMPLER_BLOCK ? 1 : 0), masked != 0, sms, largest_cluster);
+}
 extern "C" void e3_test_arm_stall(int64_t tile, uint64_t wait_ns) { e3::arm_stall(tile, wait_ns); }

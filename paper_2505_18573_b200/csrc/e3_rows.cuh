@@ -64,6 +64,8 @@ cudaError_t launch_rows(const RowsParams &p, int64_t rows, int dtype, int sample
                         cudaStream_t stream);
 
 // The kernel of short calls; taken: whether the call is one (if not, nothing has been launched).
+// Blocks per row that it gives such a call on a device of that many SMs whose largest cluster has `largest` blocks (0: not a short call).
+int direct_ctas(int64_t rows, int64_t V, int dtype, int sampler, bool mask, int sms, int largest);
 cudaError_t launch_rows_direct(const RowsParams &p, int64_t rows, int dtype, int sampler, cudaStream_t stream, bool &taken);
 
 }  // namespace e3

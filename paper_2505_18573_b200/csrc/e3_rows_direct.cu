@@ -539,20 +539,44 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) rows_direct_kernel(
 
 int64_t chunk_of(int64_t V, int64_t ctas) { return ((V + ctas - 1) / ctas + 255) / 256 * 256; }
 
+// The most CTAs of a cluster that the device can hold, each with the shared memory a CTA takes at most.  A whole B200 holds kClusterMost;
+// a partition of one (or of its SMs) may hold fewer.
+template <class K>
+int largest_cluster(K kern, int threads) {
+  for (int n = kClusterMost; n > 1; --n) {
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)n;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)n);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = kChunkBytes + kSlackBytes;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) == cudaSuccess && clusters > 0) return n;
+    cudaGetLastError();  // (no such cluster here: nobody's error)
+  }
+  return 1;
+}
+
 template <int DT, int SAMPLER, int kThreads>
-cudaError_t launch(const RowsParams &p, int64_t rows, int ctas, int dev, cudaStream_t stream) {
+cudaError_t launch(const RowsParams &p, int64_t rows, int ctas, int dev, cudaStream_t stream, bool &taken) {
   static std::mutex lock;
-  static bool ready[64];
+  static int most[64];  // CTAs of a cluster; 0: not asked yet
   auto kern = rows_direct_kernel<DT, SAMPLER, kThreads>;
   {
     std::lock_guard<std::mutex> hold(lock);
-    if (!ready[dev]) {
+    if (most[dev] == 0) {
       cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kChunkBytes + kSlackBytes);
       if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
       if (e != cudaSuccess) return e;
-      ready[dev] = true;
+      most[dev] = largest_cluster(kern, kThreads);
     }
+    if (ctas > most[dev]) return cudaSuccess;  // (the streaming kernel needs no cluster)
   }
+  taken = true;
   RowsParams q = p;
   q.wait_ns = kDefaultWaitNs;
   const int chunk = (int)chunk_of(p.V, ctas);
@@ -614,6 +638,11 @@ Plan plan(int64_t rows, int64_t V, int64_t esize, int sampler, bool mask, int64_
 
 }  // namespace
 
+int direct_ctas(int64_t rows, int64_t V, int dtype, int sampler, bool mask, int sms, int largest) {
+  const Plan w = plan(rows, V, dtype == 0 ? 4 : 2, sampler, mask, sms);
+  return w.ctas <= largest ? w.ctas : 0;
+}
+
 cudaError_t launch_rows_direct(const RowsParams &p, int64_t rows, int dtype, int sampler, cudaStream_t stream, bool &taken) {
   static std::atomic<int> sms[64];
   taken = false;
@@ -629,15 +658,14 @@ cudaError_t launch_rows_direct(const RowsParams &p, int64_t rows, int dtype, int
   }
   const Plan w = plan(rows, p.V, dtype == 0 ? 4 : 2, sampler, p.mask != nullptr, count);
   if (w.threads == 0) return cudaSuccess;
-  taken = true;
   auto go = [&](auto threads) {
     constexpr int T = decltype(threads)::value;
     if (dtype == 0) {
-      if (sampler < 0) return launch<0, -1, T>(p, rows, w.ctas, dev, stream);
-      return sampler == 0 ? launch<0, 0, T>(p, rows, w.ctas, dev, stream) : launch<0, 1, T>(p, rows, w.ctas, dev, stream);
+      if (sampler < 0) return launch<0, -1, T>(p, rows, w.ctas, dev, stream, taken);
+      return sampler == 0 ? launch<0, 0, T>(p, rows, w.ctas, dev, stream, taken) : launch<0, 1, T>(p, rows, w.ctas, dev, stream, taken);
     }
-    if (sampler < 0) return launch<1, -1, T>(p, rows, w.ctas, dev, stream);
-    return sampler == 0 ? launch<1, 0, T>(p, rows, w.ctas, dev, stream) : launch<1, 1, T>(p, rows, w.ctas, dev, stream);
+    if (sampler < 0) return launch<1, -1, T>(p, rows, w.ctas, dev, stream, taken);
+    return sampler == 0 ? launch<1, 0, T>(p, rows, w.ctas, dev, stream, taken) : launch<1, 1, T>(p, rows, w.ctas, dev, stream, taken);
   };
   return w.threads == 256 ? go(std::integral_constant<int, 256>()) : go(std::integral_constant<int, 512>());
 }

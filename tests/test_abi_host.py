@@ -31,6 +31,21 @@ def test_library_exports_every_declared_symbol(e3):
         assert hasattr(L, name), name
 
 
+@pytest.mark.parametrize("largest", [1, 2, 7, 8, 15, 16])
+def test_short_calls_keep_to_the_clusters_that_the_device_holds(e3, largest):
+    """A device that holds no cluster as large as a call asks for takes the streaming kernel; the other calls stay where they were."""
+    kinds = [(dt, sampler, masked) for dt in (e3.E3_F32, e3.E3_BF16) for sampler, masked in ((-1, False), (-1, True), (0, False), (1, False), (2, False))]
+    seen = set()
+    for dt, sampler, masked in kinds:
+        for rows in (1, 2, 4, 5, 8, 16, 33, 64, 100, 148, 300, 700, 1500, 4096):
+            for V in (1, 4096, 8000, 20001, 32000, 50257, 70000, 151936, 256000, 1 << 22):
+                whole = e3.e3_test_row_blocks(dt, rows, V, sampler, masked)
+                assert 0 <= whole <= 16
+                assert e3.e3_test_row_blocks(dt, rows, V, sampler, masked, 148, largest) == (whole if whole <= largest else 0)
+                seen.add(whole)
+    assert {0, 1, 8, 16} <= seen
+
+
 def test_status_strings_and_workspace(e3):
     assert e3.status_string(0) == "E3_OK"
     assert e3.status_string(5) == "E3_ERR_INFEASIBLE"

@@ -45,10 +45,16 @@ __device__ __forceinline__ void block_sums(double (&v)[N], double (*sh)[N]) {
   }
 }
 
-// What a part of a batch adds up: terms of the objective, tokens, clipped tokens.
+// What a thread or a warp of a batch adds up: terms of the objective, tokens, clipped tokens (an eighth of a response at most: 32 bits hold
+// what fits the device's memory).
 struct Sums {
   double terms;
-  int on, clipped;
+  uint32_t on, clipped;
+};
+// ... and a block.
+struct Totals {
+  double terms;
+  int64_t on, clipped;
 };
 __device__ __forceinline__ Sums warp_sums(Sums v) {
 #pragma unroll
@@ -58,11 +64,11 @@ __device__ __forceinline__ Sums warp_sums(Sums v) {
   return v;
 }
 // ... over the block, in a fixed order; every thread gets them.
-__device__ __forceinline__ Sums block_sums(Sums v, Sums *sh) {
-  v = warp_sums(v);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+__device__ __forceinline__ Totals block_sums(const Sums &mine, Sums *sh) {
+  const Sums warp = warp_sums(mine);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = warp;
   __syncthreads();
-  v = Sums{0.0, 0, 0};
+  Totals v = {0.0, 0, 0};
 #pragma unroll
   for (int w = 0; w < kThreads / 32; ++w) {
     v.terms += sh[w].terms;
@@ -152,8 +158,8 @@ __global__ void __launch_bounds__(kThreads) grpo_seq_kernel(const float *__restr
   const int64_t t_rest = (int64_t)threadIdx.x + kKeep * kThreads;
   Sums rest = sum;
   for (int64_t t = t_rest; t < seq_len; t += kThreads) sum.on += (!mask || mask[base + t]) ? 1 : 0;
-  sum = block_sums(sum, sh);
-  const double len = (double)sum.on, gq = sh_group;
+  Totals total = block_sums(sum, sh);
+  const double len = (double)total.on, gq = sh_group;
   const bool counts = len > 0.0 && gq > 0.0;
   const double w = counts ? 1.0 / (len * gq * (double)n_groups) : 0.0;
   if (g_out) {
@@ -176,12 +182,12 @@ __global__ void __launch_bounds__(kThreads) grpo_seq_kernel(const float *__restr
       }
       if (g_out) g_out[j] = v;
     }
-    sum = block_sums(rest, sh_rest);
+    total = block_sums(rest, sh_rest);
   }
   if (threadIdx.x == 0) {
-    part[i].J = counts ? sum.terms / (len * gq) : 0.0;
+    part[i].J = counts ? total.terms / (len * gq) : 0.0;
     part[i].tokens = gq > 0.0 ? len : 0.0;
-    part[i].clipped = counts ? (double)sum.clipped : 0.0;
+    part[i].clipped = counts ? (double)total.clipped : 0.0;
   }
 }
 
@@ -231,7 +237,7 @@ __global__ void __launch_bounds__(kShortThreads) grpo_short_kernel(const float *
       if (a <= i && i < b) group = (int)(b - a);
     }
     group = __reduce_max_sync(kAll, group);
-    Sums sum = {0.0, __popc(on), 0};
+    Sums sum = {0.0, (uint32_t)__popc(on), 0};
     double g[kShortKeep];  // gradient before the weight
 #pragma unroll
     for (int k = 0; k < kShortKeep; ++k) {

@@ -147,3 +147,13 @@ def test_grpo_objective_at_the_edges_of_one_launch(e3, sizes, seq_len, min_len):
         got = g.cpu().numpy().astype(np.float64)
         assert np.array_equal(got == 0, grad == 0)
         assert np.all(np.abs(got - grad) <= np.abs(grad) * 2.0 ** -23 + 1e-30)
+
+
+def test_grpo_objective_of_a_response_of_more_than_2_31_tokens(e3):
+    """Counts are not kept in 32 bits: with ratios of 1 the objective is the advantage, whatever the length."""
+    n = (1 << 31) + 5
+    if torch.cuda.mem_get_info()[0] < 5 * n:
+        pytest.skip("needs 11 GB of device memory")
+    logp = torch.zeros((1, n), device=DEV)
+    out, _ = e3.e3_grpo_objective(logp, logp, torch.full((1,), 0.75, device=DEV), torch.tensor([0, 1], device=DEV), want_grad=False)
+    assert out.tolist() == [0.75, 0.0]

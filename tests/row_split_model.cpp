@@ -31,7 +31,7 @@ struct Warp {
 struct Cta {
   Split p;
   Run run;
-  int sampler, next = kWarps, slow_strip, slow;
+  int next = kWarps, slow_strip, slow;
   std::vector<int> freed, owner, arrived, record;
   int piece_owner[8], piece_turn[8];
   bool piece_live[8];
@@ -84,12 +84,6 @@ struct Cta {
           x.seg = seg;
           x.count = 0;
         }
-        if (sampler == 1 && q == seg && x.count == 0) {  // the variates need the places of the whole segment
-          const int n = segment_strips(p, place(seg));
-          for (int i = 0; i < n; ++i)
-            if (freed[(q + i) & mask()] < q + i - mask()) return false;
-          ++x.count;
-        }
         if (x.n < 2 && !x.dry) take(x);
         x.until = t + (q == slow_strip ? slow : 1.0 + 0.01 * (q % 7));
         x.at = Warp::kSumming;
@@ -108,7 +102,7 @@ struct Cta {
         }
         int &a = arrived[x.seg & mask()];
         a += x.count;
-        const int need = segment_strips(p, place(x.seg)) + (sampler == 1);
+        const int need = segment_strips(p, place(x.seg));
         if (a > need) fail("count", x.seg);
         x.at = a == need ? Warp::kMerge : Warp::kIdle;
         if (a == need) {
@@ -192,7 +186,6 @@ int main(int argc, char **argv) {
     if (c.run.len > longest) longest = c.run.len;
     for (int s = b % apart; s < c.run.len; s += apart, ++plays) {
       Cta d = c;
-      d.sampler = sampler;
       d.slow_strip = s;
       d.slow = slow;
       d.play();

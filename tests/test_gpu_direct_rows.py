@@ -6,6 +6,7 @@ import torch
 import oracle
 from paper_2505_18573_b200 import inputs
 from _compare import ATOL, assert_close, assert_tokens
+from _routes import Streaming, short
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
@@ -24,6 +25,7 @@ def _check(e3, logits, temps, mask=None):
     rows, V = logits.shape
     z, t = inputs.to_oracle_array(logits), temps.cpu().numpy()
     atol = ATOL[logits.dtype]
+    assert any(short(e3, rows, V, logits.dtype, sampler) for sampler in (-1, 0, 1)) or (V == 212993 and logits.dtype == torch.float32)
     for sampler in (0, 1):
         tok, lp, en, gap = e3.e3_sample(logits, temps, 3, 1 << 34, 5, sampler, want_gap=True)
         ref = oracle.sample(z, t, 3, 1 << 34, 5, sampler)
@@ -45,7 +47,8 @@ def _check(e3, logits, temps, mask=None):
 @pytest.mark.parametrize("rows, V", [
     (3, 4095), (3, 4096), (3, 4097), (2, 65537),           # one part, two, sixteen: a last part of a few entries or of none
     (40, 16640), (40, 16641), (12, 70001),                 # parts of 256-thread blocks, of 512-thread ones; rows that begin anywhere
-    (200, 26624), (200, 53248), (7, 212993), (1, 425984),  # the longest parts
+    (200, 26624), (200, 53248), (7, 212992), (1, 425984),  # the longest parts
+    (7, 212993),                                           # ... one entry more than those of fp32 hold
     (500, 17408), (300, 35841),                            # three and four blocks of 256 threads per SM
     (900, 26001)])                                         # sampler 0: a block a row, more than two waves of them
 def test_parts(e3, dtype, rows, V):
@@ -60,6 +63,7 @@ def test_mask(e3, dtype, rows, V):
     mask = (torch.rand(rows, generator=torch.Generator().manual_seed(2)) < 0.5).to(torch.uint8).to(DEV)
     logits[mask == 0] = float("nan")  # (these are not looked at)
     temps, targets = inputs.uniform_temps(rows, seed=3, device=DEV), inputs.uniform_targets(rows, V, seed=4, device=DEV)
+    assert short(e3, rows, V, dtype, masked=True)
     total = torch.zeros(2, dtype=torch.float64, device=DEV)
     lp, en = e3.e3_token_logp_entropy(logits, targets, mask=mask, temps=temps, out_sum=total)
     rlp, ren, _ = oracle.token_logp_entropy(inputs.to_oracle_array(logits), targets.cpu().numpy(), mask=mask.cpu().numpy(), temps=temps.cpu().numpy())
@@ -80,7 +84,7 @@ def test_few_entries_and_flat_rows(e3, dtype, std):
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("V, first", [(41000, 0), (41003, 0), (41000, 1)])
 def test_same_as_the_streaming_kernel(e3, dtype, V, first):
-    """A batch for the streaming kernel and the same rows a few at a time: entries ruled out, NaN, infinities, greedy rows, temperatures
+    """A batch through the streaming kernel and the same rows a few at a time: entries ruled out, NaN, infinities, greedy rows, temperatures
     that cannot be used, rows of any alignment."""
     rows, unit = 1040, 13
     g = torch.Generator(device=DEV); g.manual_seed(V)
@@ -107,9 +111,11 @@ def test_same_as_the_streaming_kernel(e3, dtype, V, first):
     targets[::17] = V  # (not a token: no log-probability)
 
     def call(which, lo, hi):
+        way = Streaming(e3) if hi - lo == rows else e3
+        assert way is not e3 or short(e3, hi - lo, V, dtype, -1 if which is None else which)
         if which is None:
-            return e3.e3_token_logp_entropy(logits[lo:hi], targets[lo:hi], temps=temps[lo:hi], want_gap=True)
-        return e3.e3_sample(logits[lo:hi], temps[lo:hi], 11, 12, lo, which, want_gap=True)
+            return way.e3_token_logp_entropy(logits[lo:hi], targets[lo:hi], temps=temps[lo:hi], want_gap=True)
+        return way.e3_sample(logits[lo:hi], temps[lo:hi], 11, 12, lo, which, want_gap=True)
     for which in (None, 0, 1, e3.E3_SAMPLER_TOKEN_AUDIT):
         got = [t.cpu().numpy() for t in call(which, 0, rows)]
         parts = [call(which, lo, lo + 40) for lo in range(0, rows, 40)]
@@ -129,6 +135,8 @@ def test_graph_replay_on_cut_rows_of_the_streaming_kernel(e3, sampler):
     data = [inputs.zipf_gaussian_logits(rows, V, seed=80 + i, dtype=torch.bfloat16, device=DEV) for i in range(2)]
     logits, temps = data[0].clone(), inputs.uniform_temps(rows, seed=84, device=DEV)
     targets = inputs.uniform_targets(rows, V, seed=85, device=DEV)
+
+    assert not short(e3, rows, V, torch.bfloat16, -1 if sampler is None else sampler)
 
     def run(stream=None):
         if sampler is None:
@@ -156,6 +164,7 @@ def test_temperatures_that_cannot_be_used_between_others(e3, dtype):
     temps = inputs.uniform_temps(rows, seed=3, device=DEV)
     for k, bad in enumerate((-1.0, float("nan"), float("inf"))):
         temps[2 * k::6] = bad
+    assert short(e3, rows, V, dtype, 0) and short(e3, rows, V, dtype, masked=True)
     z, t = inputs.to_oracle_array(logits), temps.cpu().numpy()
     ref = oracle.sample(z, t, 3, 4, 0, 0)
     targets = inputs.uniform_targets(rows, V, seed=3, device=DEV)

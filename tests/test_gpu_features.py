@@ -10,18 +10,19 @@ import torch
 import oracle
 from paper_2505_18573_b200 import inputs
 from _compare import ATOL, assert_close
+from _routes import Streaming
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
 
 
-@pytest.fixture(scope="module")
-def e3():
+@pytest.fixture(scope="module", params=["routed", "streaming"])
+def e3(request):
     if not torch.cuda.is_available():
         pytest.skip("needs a CUDA device")
     from paper_2505_18573_b200 import binding
     binding.lib()   # raises when the CUDA library has not been built: no fallback
-    return binding
+    return Streaming(binding) if request.param == "streaming" else binding
 
 
 # ----------------------------------------------------------------------------------------------

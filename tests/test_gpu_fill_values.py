@@ -7,7 +7,7 @@ import torch
 import oracle
 from paper_2505_18573_b200 import inputs
 from _compare import ATOL, assert_close, assert_tokens
-from _routes import streaming
+from _routes import Streaming, short
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
@@ -50,13 +50,16 @@ def _rows(V, dtype):
 def test_runs_of_a_fill_value(e3, dtype, V, kernel):
     logits = (_rows(V, dtype) if V > 16384 else _rows(20001, dtype)[:, 18001:].contiguous()).to(DEV)
     rows, atol = len(logits), ATOL[dtype]
-    call = streaming(e3) if kernel == "streaming" else lambda f, *a, **k: f(*a, **k)
+    if kernel == "streaming":
+        e3 = Streaming(e3)
+    else:
+        assert all(short(e3, rows, V, dtype, sampler) for sampler in (-1, 0, 1, 2))
     for tau in (1.0, 0.61, 0.87, 1.37):
         temps = torch.full((rows,), tau, device=DEV)
         z, t = inputs.to_oracle_array(logits), temps.cpu().numpy()
         gap = oracle.row_gap(z, t)
         for sampler in (0, 1, e3.E3_SAMPLER_TOKEN_AUDIT):
-            tok, lp, en, gp = call(e3.e3_sample, logits, temps, 3, 9, 5, sampler, want_gap=True)
+            tok, lp, en, gp = e3.e3_sample(logits, temps, 3, 9, 5, sampler, want_gap=True)
             ref = oracle.sample(z, t, 3, 9, 5, sampler % 2)
             tok = tok.cpu().numpy()
             assert_tokens(f"tau{tau}s{sampler}", tok, ref, sampler)
@@ -65,14 +68,14 @@ def test_runs_of_a_fill_value(e3, dtype, V, kernel):
             assert_close("logp", lp.cpu().numpy()[same], ref.logp[same], atol)
             assert_close("gap", gp.cpu().numpy(), gap, atol)
         targets = logits.float().argmax(1).to(torch.int32)
-        lp, en, gp = call(e3.e3_token_logp_entropy, logits, targets, temps=temps, want_gap=True)
+        lp, en, gp = e3.e3_token_logp_entropy(logits, targets, temps=temps, want_gap=True)
         rlp, ren, _ = oracle.token_logp_entropy(z, targets.cpu().numpy(), temps=t)
         assert_close("train.logp", lp.cpu().numpy(), rlp, atol)
         assert_close("train.ent", en.cpu().numpy(), ren, atol)
         assert_close("train.gap", gp.cpu().numpy(), gap, atol)
         # entries of the fill value as targets: the division by tau and the product with its reciprocal round once each
         targets = logits.float().argmin(1).to(torch.int32)
-        lp, _ = call(e3.e3_token_logp_entropy, logits, targets, temps=temps)
+        lp, _ = e3.e3_token_logp_entropy(logits, targets, temps=temps)
         rlp = oracle.token_logp_entropy(z, targets.cpu().numpy(), temps=t)[0]
         ok = np.abs(rlp) < 3e38
         assert_close("fill.logp", lp.cpu().numpy()[ok] / np.maximum(1, np.abs(rlp[ok])), rlp[ok] / np.maximum(1, np.abs(rlp[ok])), atol)

@@ -1,4 +1,5 @@
-"""The row kernel and the entropy mean at the edges of their splits, against the fp64 oracle (tolerances of `_compare`)."""
+"""The streaming row kernel (every row call here goes through it) and the entropy mean at the edges of their splits, against the fp64
+oracle (tolerances of `_compare`)."""
 import numpy as np
 import pytest
 import torch
@@ -6,6 +7,7 @@ import torch
 import oracle
 from paper_2505_18573_b200 import inputs
 from _compare import ATOL, assert_close, assert_tokens
+from _routes import Streaming
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
@@ -17,7 +19,7 @@ def e3():
         pytest.skip("needs a CUDA device")
     from paper_2505_18573_b200 import binding
     binding.lib()
-    return binding
+    return Streaming(binding)
 
 
 def _check(e3, logits, temps, samplers=(0, 1), mask=None, workspace=None):
@@ -43,7 +45,7 @@ def _check(e3, logits, temps, samplers=(0, 1), mask=None, workspace=None):
     (5, 1024), (37, 2049), (149, 6145),   # one tile a row, a tile and an entry, three tiles and an entry
     (17, 101000), (100, 101000),          # one strip per warp of 1 and of a few tiles
     (290, 101000), (600, 33333),          # ... of a few tiles more, most warps busy; rows that begin anywhere
-    (700, 65001)])                        # strips of 8 tiles and more than one per warp
+    (700, 65001)])                        # more than one strip per warp
 def test_strip_lengths(e3, dtype, rows, V):
     logits = inputs.zipf_gaussian_logits(rows, V, seed=rows, dtype=dtype, device=DEV)
     _check(e3, logits, inputs.uniform_temps(rows, seed=V, device=DEV))
@@ -57,13 +59,14 @@ def test_strips_of_the_statistics(e3, dtype, rows, V):
 
 
 @pytest.mark.parametrize("sampler, dtype, rows, V", [
-    (None, torch.bfloat16, 9000, 70001), (None, torch.bfloat16, 600, 1200001),  # rows of 5 strips, of several segments
-    (1, torch.bfloat16, 2500, 70001), (1, torch.bfloat16, 4000, 70001),         # strips of 8 tiles, of 4
-    (1, torch.float32, 400, 300001), (1, torch.float32, 200, 700001),           # pieces of two segments, of three
-    (0, torch.bfloat16, 16000, 70001)])
+    (None, torch.bfloat16, 9000, 70001), (None, torch.bfloat16, 600, 1200001),  # runs of 305 strips, rows of 5 and 74 of 8 tiles
+    (None, torch.bfloat16, 300, 2200001), (1, torch.float32, 250, 1300001),     # ... of 270, rows of two segments
+    (1, torch.bfloat16, 9000, 70001), (0, torch.bfloat16, 20000, 70001),        # ... of 305, of 271 with rows of two strips of 25
+    (1, torch.bfloat16, 2500, 70001), (1, torch.bfloat16, 4000, 70001), (1, torch.float32, 400, 300001),  # shorter runs than the ring
+    (1, torch.float32, 200, 700001), (0, torch.bfloat16, 16000, 70001)])
 def test_runs_longer_than_the_ring(e3, sampler, dtype, rows, V):
-    """More strips in a block's run than it keeps records of, rows that begin anywhere: the same as in batches of a few rows, where
-    no warp takes a second strip."""
+    """More strips in a block's run than the 256 it keeps records of (and nearly as many), rows that begin anywhere: the same as in
+    batches of a few rows, where no warp takes a second strip."""
     g = torch.Generator(device=DEV); g.manual_seed(rows)
     logits = torch.empty((rows, V), dtype=dtype, device=DEV)
     for lo in range(0, rows, 500):
@@ -96,9 +99,10 @@ def test_whole_rows_of_several_segments(e3, dtype, V):
     _check(e3, logits, inputs.uniform_temps(3, seed=1, device=DEV), samplers=(0,), workspace=tiny)
 
 
-def test_blocked_sampler_rows_longer_than_its_half_ring(e3):
-    """Rows of several segments in a run that still fits the ring."""
-    rows, V = 140, 400001
+@pytest.mark.parametrize("rows, V", [(140, 400001),    # 25 strips of 16 tiles a row
+                                     (148, 1080001)])  # 132 strips of 8 tiles a row, which a block holds whole
+def test_blocked_sampler_rows_longer_than_its_half_ring(e3, rows, V):
+    """Long rows, also of several segments, in a run that still fits the ring."""
     logits = inputs.zipf_gaussian_logits(rows, V, seed=9, dtype=torch.float32, device=DEV)
     _check(e3, logits, inputs.uniform_temps(rows, seed=2, device=DEV), samplers=(1,))
 

@@ -5,6 +5,8 @@ import gc
 import pytest
 import torch
 
+from _routes import Streaming
+
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
 
@@ -15,7 +17,7 @@ def e3():
         pytest.skip("needs a CUDA device")
     from paper_2505_18573_b200 import binding
     binding.lib()
-    return binding
+    return Streaming(binding)  # (the kernel of short calls has no use for scratch)
 
 
 class _Calls:
@@ -38,6 +40,13 @@ class _Calls:
 
     def clear(self):
         self.tok.fill_(-7); self.logp.zero_(); self.ent.zero_()
+
+
+def test_the_calls_here_write_their_scratch(e3):
+    for calls in (_Calls(e3), _Calls(e3, 3), _Calls(e3, 8), _Calls(e3, 40, 150000), _Calls(e3, 700)):
+        room = torch.full((calls.need,), 0x5A, dtype=torch.uint8, device=DEV)
+        e3.e3_sample(calls.logits, calls.temps, 3, 4, sampler=e3.E3_SAMPLER_BLOCK, workspace=room)
+        assert bool((room != 0x5A).any())
 
 
 def _canaries(stream, nbytes):

@@ -1124,9 +1124,11 @@ void arm_stall(int64_t stall_tile, unsigned long long wait_ns) {
 cudaError_t launch_rows(const RowsParams &p, int64_t rows, int dtype, int sampler, void *workspace, size_t workspace_bytes,
                         cudaStream_t stream) {
   if ((dtype != 0 && dtype != 1) || sampler < -1 || sampler > 1) return cudaErrorInvalidValue;
-  if (g_stall_tile.load() < 0) {  // (the hook stalls a tile of the streaming kernel)
+  long long stall = g_stall_tile.load();
+  if (stall < 0) {  // (else the hook stalls a tile of the streaming kernel)
+    if (stall < -1) stall = g_stall_tile.exchange(-1);
     bool taken = false;
-    const cudaError_t e = launch_rows_direct(p, rows, dtype, sampler, stream, taken);
+    const cudaError_t e = launch_rows_direct(p, rows, dtype, sampler, BlockStall{-2 - stall, g_stall_wait_ns.load()}, stream, taken);
     if (taken || e != cudaSuccess) return e;
   }
   if (dtype == 0) {

@@ -477,7 +477,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) rows_direct_kernel(
   }
   if (SAMPLER == 0 && pc.tb[0] >= 0) pc.zf = lds_elem<DT>(base + a + (uint32_t)((pc.tb[0] - e0) * F::kEsize));
   if (ctas > 1) {
-    if (lane < 4) {
+    if (lane < 4 && row_ptr(p, row) + (size_t)e0 * F::kEsize != p.stall_src) {
       const float x0 = lane == 0 ? pc.M : (lane == 1 ? pc.ty[0] : (lane == 2 ? __int_as_float(pc.tb[0]) : pc.zf));
       const float x1 = lane == 0 ? pc.Z : (lane == 1 ? pc.ty[1] : (lane == 2 ? __int_as_float(pc.tb[1]) : 0.f));
       const float x2 = lane == 0 ? pc.W : (lane == 1 ? pc.ty[2] : (lane == 2 ? __int_as_float(pc.tb[2]) : 0.f));
@@ -563,7 +563,7 @@ int largest_cluster(K kern, int threads) {
 }
 
 template <int DT, int SAMPLER, int kThreads>
-cudaError_t launch(const RowsParams &p, int64_t rows, int ctas, int dev, cudaStream_t stream, bool &taken) {
+cudaError_t launch(const RowsParams &p, int64_t rows, int ctas, int dev, const BlockStall &stall, cudaStream_t stream, bool &taken) {
   static std::mutex lock;
   static int most[64];  // CTAs of a cluster; 0: not asked yet
   auto kern = rows_direct_kernel<DT, SAMPLER, kThreads>;
@@ -579,8 +579,13 @@ cudaError_t launch(const RowsParams &p, int64_t rows, int ctas, int dev, cudaStr
   }
   taken = true;
   RowsParams q = p;
-  q.wait_ns = kDefaultWaitNs;
   const int chunk = (int)chunk_of(p.V, ctas);
+  q.wait_ns = kDefaultWaitNs;
+  q.stall_src = nullptr;
+  if (stall.block >= 0) {
+    q.wait_ns = stall.wait_ns;
+    q.stall_src = p.logits + stall.block / ctas * p.row_bytes + stall.block % ctas * chunk * Fmt<DT>::kEsize;
+  }
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -662,7 +667,7 @@ int direct_ctas(int64_t rows, int64_t V, int dtype, int sampler, bool mask, int 
   return w.ctas <= largest ? w.ctas : 0;
 }
 
-cudaError_t launch_rows_direct(const RowsParams &p, int64_t rows, int dtype, int sampler, cudaStream_t stream, bool &taken) {
+cudaError_t launch_rows_direct(const RowsParams &p, int64_t rows, int dtype, int sampler, const BlockStall &stall, cudaStream_t stream, bool &taken) {
   static std::atomic<int> sms[64];
   taken = false;
   int dev = 0;
@@ -680,11 +685,11 @@ cudaError_t launch_rows_direct(const RowsParams &p, int64_t rows, int dtype, int
   auto go = [&](auto threads) {
     constexpr int T = decltype(threads)::value;
     if (dtype == 0) {
-      if (sampler < 0) return launch<0, -1, T>(p, rows, w.ctas, dev, stream, taken);
-      return sampler == 0 ? launch<0, 0, T>(p, rows, w.ctas, dev, stream, taken) : launch<0, 1, T>(p, rows, w.ctas, dev, stream, taken);
+      if (sampler < 0) return launch<0, -1, T>(p, rows, w.ctas, dev, stall, stream, taken);
+      return sampler == 0 ? launch<0, 0, T>(p, rows, w.ctas, dev, stall, stream, taken) : launch<0, 1, T>(p, rows, w.ctas, dev, stall, stream, taken);
     }
-    if (sampler < 0) return launch<1, -1, T>(p, rows, w.ctas, dev, stream, taken);
-    return sampler == 0 ? launch<1, 0, T>(p, rows, w.ctas, dev, stream, taken) : launch<1, 1, T>(p, rows, w.ctas, dev, stream, taken);
+    if (sampler < 0) return launch<1, -1, T>(p, rows, w.ctas, dev, stall, stream, taken);
+    return sampler == 0 ? launch<1, 0, T>(p, rows, w.ctas, dev, stall, stream, taken) : launch<1, 1, T>(p, rows, w.ctas, dev, stall, stream, taken);
   };
   return w.threads == 256 ? go(std::integral_constant<int, 256>()) : go(std::integral_constant<int, 512>());
 }

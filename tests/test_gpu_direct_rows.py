@@ -177,3 +177,31 @@ def test_temperatures_that_cannot_be_used_between_others(e3, dtype):
         lp, en = e3.e3_token_logp_entropy(logits, targets, mask=mask, temps=temps)
         assert_close("train.logp", lp.cpu().numpy(), rlp, ATOL[dtype])
         assert_close("train.ent", en.cpu().numpy(), ren, ATOL[dtype])
+
+
+@pytest.mark.parametrize("rows, V, block", [(6, 151936, 2 * 8 + 3), (6, 151936, 5 * 8), (1, 151936, 15), (100, 20001, 99 * 2 + 1)])
+@pytest.mark.parametrize("sampler", [None, 0, 1])
+def test_a_part_that_is_never_handed_over(e3, sampler, rows, V, block):
+    """The wait for it runs out: the row reads NaN, the status word says so, the other rows and the next call are as ever."""
+    ctas = short(e3, rows, V, torch.bfloat16, -1 if sampler is None else sampler)
+    assert ctas > 1
+    row = block // ctas
+    logits = inputs.zipf_gaussian_logits(rows, V, seed=5, dtype=torch.bfloat16, device=DEV)
+    temps, targets = inputs.uniform_temps(rows, seed=6, device=DEV), inputs.uniform_targets(rows, V, seed=7, device=DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+
+    def run():
+        if sampler is None:
+            return e3.e3_token_logp_entropy(logits, targets, temps=temps, status=status)
+        return e3.e3_sample(logits, temps, 3, 4, 0, sampler, status=status)
+    want = run()
+    assert int(status[0]) == 0
+    e3.e3_test_arm_stall(-2 - block, 5_000_000)  # 5 ms instead of two seconds
+    got = run()
+    assert int(status[0]) == e3.E3_STATUS_TIMEOUT
+    others = torch.arange(rows, device=DEV) != row
+    for g, w in zip(got, want):
+        assert torch.equal(g[others], w[others])
+        assert int(g[row]) == -1 if g.dtype == torch.int32 else bool(torch.isnan(g[row]))
+    status.zero_()
+    assert all(torch.equal(a, b) for a, b in zip(run(), want)) and int(status[0]) == 0

@@ -78,7 +78,9 @@ constexpr int kThreads = kWarps * 32;
 constexpr int kStages = 2;       // ring slots per warp
 constexpr int kMaxLive = 1024;   // rows of a CTA's run with a response mask (their numbers are kept in shared memory)
 constexpr int kQueueCap = 64;    // sampler 0: a push meets at most 31 entries and adds at most 32
-constexpr int kStripBlocks = kBlockStripTiles * 8;  // sampler 1: most blocks of a strip
+constexpr int kStripBlocks = longest_strip(1, true) * Fmt<1>::kBT;  // sampler 1: most blocks of a strip
+static_assert(longest_strip(1, false) * Fmt<0>::kBT <= kStripBlocks && kLongRunStrip <= longest_strip(1, true) && kLongRunStrip <= longest_strip(1, false),
+              "room for the blocks of every strip");
 
 // An entry of sampler 0 that may win: vocabulary index (with kAnyByte: its coarse byte has not been looked at, else it is
 // 255) and logit.
@@ -187,6 +189,28 @@ __device__ __forceinline__ int read_best(const u64 *bests, int seg) {
 // ---------------------------------------------------------------------------------------------
 // Row results
 // ---------------------------------------------------------------------------------------------
+__device__ __forceinline__ void piece_reset(Piece &pc) {
+  pc.M = pc.Z = pc.W = pc.zf = 0.f;
+  pc.err = 0;
+  pc.zmax = -CUDART_INF_F;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) { pc.ty[i] = -CUDART_INF_F; pc.tb[i] = -1; }
+}
+// Merges q into pc.
+__device__ __forceinline__ void piece_merge(Piece &pc, const Piece &q) {
+  pc.err |= q.err;
+  pc.zmax = fmaxf(pc.zmax, q.zmax);
+  merge_stats_f(pc.M, pc.Z, pc.W, q.M, q.Z, q.W);
+  Top3 top;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) { top.y[i] = pc.ty[i]; top.b[i] = pc.tb[i]; }
+  if (q.tb[0] >= 0 && best_before(q.ty[0], q.tb[0], top.y[0], top.b[0])) pc.zf = q.zf;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) top3_insert(top, q.ty[i], q.tb[i]);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) { pc.ty[i] = top.y[i]; pc.tb[i] = top.b[i]; }
+}
+
 // A row piece of this CTA is complete (all lanes hold the same pc): finishes the row, or, when the row is cut, publishes
 // the piece and finishes the row if the other pieces are all there.
 template <int DT, int SAMPLER>
@@ -353,6 +377,42 @@ __device__ __noinline__ void mark_unfinished(const uint32_t *live_rows) {
 // ---------------------------------------------------------------------------------------------
 // Samplers
 // ---------------------------------------------------------------------------------------------
+// Enters (y, b) in a list of three leaders (a warp's or a segment's); zf follows the first.  One lane.
+template <class L>
+__device__ __forceinline__ void lead_insert(L &ws, float y, int b, float z) {
+  if (top3_before(y, b, ws.ty[0], ws.tb[0])) {
+    ws.ty[2] = ws.ty[1]; ws.tb[2] = ws.tb[1]; ws.ty[1] = ws.ty[0]; ws.tb[1] = ws.tb[0]; ws.ty[0] = y; ws.tb[0] = b;
+    ws.zf = z;
+  } else if (top3_before(y, b, ws.ty[1], ws.tb[1])) {
+    ws.ty[2] = ws.ty[1]; ws.tb[2] = ws.tb[1]; ws.ty[1] = y; ws.tb[1] = b;
+  } else if (top3_before(y, b, ws.ty[2], ws.tb[2])) {
+    ws.ty[2] = y; ws.tb[2] = b;
+  }
+}
+
+// Enters the lanes' scored candidates (y, i; logit z) that may win in a list of leaders.  best: encoded lower bound of the best score
+// (the same in all lanes); returns it, raised.
+template <class L>
+__device__ __forceinline__ int enter_leaders(L &ws, bool valid, float y, int i, float z, int best, float slack_scale) {
+  constexpr unsigned kAll = 0xffffffffu;
+#pragma unroll 1
+  for (;;) {
+    valid = valid && y >= dec_float(best);  // else more than two slacks below a score already seen (or NaN)
+    if (!__any_sync(kAll, valid)) break;
+    const int e = valid ? enc_float(y) : INT_MIN, emax = __reduce_max_sync(kAll, e);
+    const int imin = __reduce_min_sync(kAll, valid && e == emax ? i : INT_MAX);
+    if (valid && e == emax && i == imin) {
+      lead_insert(ws, y, i, z);
+      valid = false;
+    }
+    __syncwarp();
+    const float ym = dec_float(emax);
+    const int enc = enc_float(ym - 4.f * score_slack(ym, slack_scale) - 2e-7f * fabsf(ym));
+    best = enc > best ? enc : best;
+  }
+  return best;
+}
+
 // Enters a warp's leaders in its segment's list.  One lane; the list is locked for the few instructions this takes.  False
 // when the wait for the lock ran out.
 __device__ __noinline__ bool hand_in_leaders(int seg) {
@@ -1057,7 +1117,7 @@ cudaError_t launch_one(RowsParams p, int64_t rows, void *workspace, size_t works
   p.spr = (int)spr;
   p.inv_spr = 1.0f / (float)spr;
   p.unit = can_cut ? 1 : (int)spr;
-  p.ring = ring_strips((int)strip, SAMPLER);
+  p.ring = kRing;
   p.ws_pieces = can_cut ? static_cast<unsigned char *>(workspace) : nullptr;
   p.wait_ns = kDefaultWaitNs;
   const long long stall = g_stall_tile.exchange(-1);  // (row * tpr + tile within the row)

@@ -1130,42 +1130,6 @@ __device__ __noinline__ int settle_exact(const EvalCtx &x, const Top3 &top, floa
   return ibest;
 }
 
-// Enters (y, b) in a list of three leaders (a warp's or a segment's); zf follows the first.  One lane.
-template <class L>
-__device__ __forceinline__ void lead_insert(L &ws, float y, int b, float z) {
-  if (top3_before(y, b, ws.ty[0], ws.tb[0])) {
-    ws.ty[2] = ws.ty[1]; ws.tb[2] = ws.tb[1]; ws.ty[1] = ws.ty[0]; ws.tb[1] = ws.tb[0]; ws.ty[0] = y; ws.tb[0] = b;
-    ws.zf = z;
-  } else if (top3_before(y, b, ws.ty[1], ws.tb[1])) {
-    ws.ty[2] = ws.ty[1]; ws.tb[2] = ws.tb[1]; ws.ty[1] = y; ws.tb[1] = b;
-  } else if (top3_before(y, b, ws.ty[2], ws.tb[2])) {
-    ws.ty[2] = y; ws.tb[2] = b;
-  }
-}
-
-// Enters the lanes' scored candidates (y, i; logit z) that may win in a list of leaders.  best: encoded lower bound of the best score
-// (the same in all lanes); returns it, raised.
-template <class L>
-__device__ __forceinline__ int enter_leaders(L &ws, bool valid, float y, int i, float z, int best, float slack_scale) {
-  constexpr unsigned kAll = 0xffffffffu;
-#pragma unroll 1
-  for (;;) {
-    valid = valid && y >= dec_float(best);  // else more than two slacks below a score already seen (or NaN)
-    if (!__any_sync(kAll, valid)) break;
-    const int e = valid ? enc_float(y) : INT_MIN, emax = __reduce_max_sync(kAll, e);
-    const int imin = __reduce_min_sync(kAll, valid && e == emax ? i : INT_MAX);
-    if (valid && e == emax && i == imin) {
-      lead_insert(ws, y, i, z);
-      valid = false;
-    }
-    __syncwarp();
-    const float ym = dec_float(emax);
-    const int enc = enc_float(ym - 4.f * score_slack(ym, slack_scale) - 2e-7f * fabsf(ym));
-    best = enc > best ? enc : best;
-  }
-  return best;
-}
-
 __device__ __forceinline__ const char *row_ptr(const RowsParams &p, uint32_t row) { return p.logits + (size_t)row * (size_t)p.row_bytes; }
 
 // ---------------------------------------------------------------------------------------------
@@ -1217,28 +1181,6 @@ __device__ __forceinline__ void write_plain(const RowsParams &p, uint32_t row, f
   if (p.out_logp) p.out_logp[row] = v;
   if (p.out_ent) p.out_ent[row] = v;
   if (p.out_gap) p.out_gap[row] = v;
-}
-
-__device__ __forceinline__ void piece_reset(Piece &pc) {
-  pc.M = pc.Z = pc.W = pc.zf = 0.f;
-  pc.err = 0;
-  pc.zmax = -CUDART_INF_F;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) { pc.ty[i] = -CUDART_INF_F; pc.tb[i] = -1; }
-}
-// Merges q into pc.
-__device__ __forceinline__ void piece_merge(Piece &pc, const Piece &q) {
-  pc.err |= q.err;
-  pc.zmax = fmaxf(pc.zmax, q.zmax);
-  merge_stats_f(pc.M, pc.Z, pc.W, q.M, q.Z, q.W);
-  Top3 top;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) { top.y[i] = pc.ty[i]; top.b[i] = pc.tb[i]; }
-  if (q.tb[0] >= 0 && best_before(q.ty[0], q.tb[0], top.y[0], top.b[0])) pc.zf = q.zf;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) top3_insert(top, q.ty[i], q.tb[i]);
-#pragma unroll
-  for (int i = 0; i < 3; ++i) { pc.ty[i] = top.y[i]; pc.tb[i] = top.b[i]; }
 }
 
 }  // namespace

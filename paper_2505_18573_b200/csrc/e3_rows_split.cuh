@@ -14,8 +14,10 @@ namespace e3 {
 namespace {
 
 constexpr int kWarps = 24;           // one CTA per SM: 80 registers a thread
-constexpr int kRing = 256;           // most strips whose records the CTA keeps (RowsParams::ring of them are)
-constexpr int kBlockStripTiles = 13;  // sampler 1: most tiles of a strip
+constexpr int kRing = 256;           // strips whose records the CTA keeps (RowsParams::ring)
+// Most tiles of a strip: of the statistics (sampler -1), of sampler 0, of sampler 1.
+constexpr int longest_strip(int sampler, bool bf16) { return sampler == 0 ? 25 : (bf16 ? (sampler == 1 ? 13 : 14) : 24); }
+constexpr int kLongRunStrip = 8;  // ... of runs of many strips per warp (but for sampler 0)
 
 // The CTA's run of strips, numbered q = 0..len-1 in hand-out order: vocabulary order, except that the strips of the last row
 // come first when that row is cut.
@@ -121,16 +123,13 @@ E3_SPLIT int long_piece_place(const Place &w) {
 // that: 4,096 rows 12 tiles 537, 25 tiles 494; sampler 1, 4,096 rows 4, 6, 8, 12 tiles 245, 230, 221, 230, 1,024 rows 72, 69, 67, 67).
 inline int strip_tiles(int64_t rows, int64_t tpr, int64_t ctas, int sampler, int tile_entries) {
   const int64_t warps = ctas * kWarps, per_warp = rows * tpr / warps;
-  const int64_t longest = sampler == 0 ? 25 : (tile_entries > 1024 ? (sampler == 1 ? 13 : 14) : 24);
+  const int64_t longest = longest_strip(sampler, tile_entries > 1024);
   for (int64_t n = per_warp < 1 ? 1 : per_warp; n <= longest; ++n) {
     const int64_t spr = (tpr + n - 1) / n, last = tpr - (spr - 1) * n, more = rows * spr - warps;
     if (more <= 0 || (sampler != 0 && n >= 8 && 2 * last <= n && more <= warps / 64)) return (int)n;
   }
-  if (sampler == 0) return 25;
-  return 8;
+  return sampler == 0 ? (int)longest : kLongRunStrip;
 }
-// Strips whose records a CTA keeps (whatever their length and the sampler).
-inline int ring_strips(int /*strip*/, int /*sampler*/) { return kRing; }
 
 }  // namespace
 }  // namespace e3

@@ -175,7 +175,7 @@ int main(int argc, char **argv) {
   Split p;
   p.spr = (int)((tpr + strip - 1) / strip);
   p.unit = 1;
-  p.ring = ring_strips(strip, sampler);
+  p.ring = kRing;
   p.inv_spr = 1.0f / (float)p.spr;
   long faults = 0, plays = 0;
   int longest = 0;

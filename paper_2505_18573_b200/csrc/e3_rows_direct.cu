@@ -19,7 +19,6 @@
 // fp32 13.5, 6.2.
 #include "e3_rows.cuh"
 #include "e3_rows_device.cuh"
-#include "e3_rows_split.cuh"
 
 #include <atomic>
 #include <mutex>
@@ -612,19 +611,19 @@ cudaError_t launch(const RowsParams &p, int64_t rows, int ctas, int dev, const B
 // borne by rows of one block (blocked sampler 645 x 24,384 bf16, 109 % of a wave, 18.4 (21.4)); of two blocks with the statistics, and not with the
 // blocked sampler, which has more to do behind its sums (226 x 55,552 bf16, 102 %, 20.6 (18.5); 223 x 28,416 fp32, 100 %, 15.2 (16.7)); of three
 // and more, which do not fill the SMs to the last place, with the statistics of fp32 (119 x 57,434, 107 %, 13.2 (14.7)) and where an SM holds four
-// blocks (104 x 150,592 bf16, 105 %, 13.4 (14.9)), else up to a full wave (87 x 160,036, 98 %, 15.7 (16.1); 155 x 91,282 in three parts, 105 %, 17.1 (16.4), in four, four to an SM,
-// 13.9); with the blocked sampler well below one (171 x 74,368, 87 %, 16.8 (17.5); 78 x 169,646, 88 %, 20.2 (19.3); 82 x 177,472, 92 %, 23.9
-// (17.9); 160 x 100,000, 108 %, 26.0 (18.6)).
+// blocks (104 x 150,592 bf16, 105 %, 13.4 (14.9)), else up to a full wave (87 x 160,036, 98 %, 15.7 (16.1); 155 x 91,282 in three
+// parts, 105 %, 17.1 (16.4), in four, four to an SM, 13.9); with the blocked sampler well below one (171 x 74,368, 87 %, 16.8 (17.5); 78 x 169,646,
+// 88 %, 20.2 (19.3); 82 x 177,472, 92 %, 23.9 (17.9); 160 x 100,000, 108 %, 26.0 (18.6)).
 // Sampler 0 gains more here than a second wave costs: 1,000 x 20,000 31.6 (48.6), 128 x 151,936 35.9 (41.7), 256 x 151,936 62.2 (57.5).
 // Of the CTAs of a call with a response mask many have nothing to do, and which is not known here: the lines lie where the kernels are even
 // with seven or eight rows of ten unmasked (us with six, eight and all ten).  Two parts a row 1,010 x 43,712 bf16 (3.4 waves) 19.6 (21.7), 23.5
 // (24.9), 27.0 (25.2), 862 x 67,984 (3.9) 25.1 (24.2), 31.2 (27.2), 35.5 (30.2); three 386 x 94,683 (2.6) 21.8 (24.9), 26.1 (27.0), 29.8 (29.5),
 // 404 x 103,568 (2.7) 20.7 (21.6), 25.2 (23.9), 28.3 (25.9); fp32 four parts 379 x 54,976 (3.4) 17.0 (18.8), 20.2 (21.6), 22.9 (23.9).
 // Where one block takes a whole row of 32 KB or more, more waves still pay: five with a mask (1,250 x 40,000 bf16 20.4 (23.7), all rows
-// 28.3 (30.6); 2,400 x 35,000, 5.4 waves, 30.8 (29.7), 44.7 (42.2); 1,500 x 50,000, 5.1, 27.9 (29.3), 39.8 (37.7)), and seven of rows up to 64 KB
-// in fp32 (3,049 x 8,320, 5.2 waves, 17.4 (19.7), 24.0 (26.5)) or whose strips would be more than one per warp of the streaming kernel (4,096 x
-// 20,000 bf16, 6.9, 29.2 (30.6), 41.7 (43.3); one strip per warp: 3,500 x 17,000, 5.9, 24.4 (24.4), 34.4 (32.4)), but not 8,192 x 32,000 87.1
-// (71.3).  Sampler 0: four, 1,500 x 32,000 63.5 (72.1), but 3,000 x 32,000 116 (113).  Without a mask the streaming kernel has no mask to count.
+// 28.3 (30.6); 2,400 x 35,000, 5.4 waves, 30.8 (29.7), 44.7 (42.2); 1,500 x 50,000, 5.1, 27.9 (29.3), 39.8 (37.7)), and seven of rows up to 64
+// KB (4,096 x 20,000 bf16, 6.9, 29.2 (30.6), 41.7 (43.3), 3,255 x 19,520, 5.5, with 57 rows of a hundred 24.9 (28.0); 3,500 x 17,000, 5.9, 24.4
+// (24.4), but all rows 34.4 (32.4)), not 8,192 x 32,000 87.1 (71.3).  Sampler 0: four, 1,500 x 32,000
+// 63.5 (72.1), but 3,000 x 32,000 116 (113).  Without a mask the streaming kernel has no mask to count.
 struct Plan {
   int threads, ctas;
 };
@@ -652,9 +651,7 @@ Plan plan(int64_t rows, int64_t V, int64_t esize, int sampler, bool mask, int64_
   if ((mask || sampler == 0) && row >= 32 * 1024 && row <= kChunkBytes) {
     const int64_t threads = row <= 70 * 1024 ? 256 : 512, fit = 227 * 1024 / (row + 6 * 1024);
     const int64_t per_sm = fit < 1024 / threads ? fit : 1024 / threads;
-    const int64_t tile = kTileBytes / esize, tpr = (V + tile - 1) / tile;
-    const int64_t strip = strip_tiles(rows, tpr, sms, -1, (int)tile), strips = rows * ((tpr + strip - 1) / strip);
-    const int64_t waves = sampler == 0 ? 4 : (row <= 64 * 1024 && (esize == 4 || strips > sms * kWarps) ? 7 : 5);
+    const int64_t waves = sampler == 0 ? 4 : (row <= 64 * 1024 ? 7 : 5);
     if (rows <= waves * per_sm * sms) return Plan{(int)threads, 1};
   }
   return Plan{0, 0};

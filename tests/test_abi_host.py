@@ -50,7 +50,7 @@ def test_short_calls_keep_to_the_clusters_that_the_device_holds(e3, largest):
     ("bf16", 160, 100000, 1, False, False), ("bf16", 82, 177472, 1, False, False), ("bf16", 226, 55552, 1, False, False),  # blocked, behind its lines
     ("bf16", 171, 74368, 1, False, True), ("bf16", 222, 54521, 1, False, True), ("bf16", 645, 24384, 1, False, True),     # ... before them
     ("bf16", 150, 100000, -1, False, True), ("bf16", 67, 224064, -1, False, False), ("fp32", 119, 57434, -1, False, True),
-    ("bf16", 2400, 35000, -1, True, False), ("bf16", 1500, 50000, -1, True, False), ("bf16", 3500, 17000, -1, True, False),
+    ("bf16", 2400, 35000, -1, True, False), ("bf16", 1500, 50000, -1, True, False), ("bf16", 3255, 19520, -1, True, True),
     ("bf16", 4096, 20000, -1, True, True), ("fp32", 3049, 8320, -1, True, True), ("bf16", 862, 67984, -1, True, False),
     ("bf16", 1010, 43712, -1, True, True), ("bf16", 404, 103568, -1, True, False), ("bf16", 386, 94683, -1, True, True),
     ("bf16", 1184, 41000, 0, False, True), ("bf16", 1300, 41000, 0, False, False)])

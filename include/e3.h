@@ -384,8 +384,8 @@ E3_API double e3_anneal_target(const e3_sched *s);
  * The consumer of that tile then runs into the bounded wait: the call returns as usual, the rows of the
  * thread block concerned read token -1 / NaN, and E3_STATUS_TIMEOUT appears in the status word.  One shot.
  * tile >= 0 sends the call to the streaming kernel (a tile behind the call's last one stalls nothing), -1 disarms the hook; from -2 on
- * down a short call (see e3_test_row_blocks) whose rows have several blocks lacks the part of block -2 - tile (row * blocks per
- * row + block), and that row is given up on in the same way.
+ * down row -2 - tile of a short call (see e3_test_row_blocks) whose rows have several blocks waits for a part that never comes, and
+ * is given up on in the same way.
  */
 E3_API void e3_test_arm_stall(int64_t tile, uint64_t wait_ns);
 

@@ -297,7 +297,7 @@ def e3_test_row_blocks(dt: int, rows: int, V: int, sampler: int = -1, masked: bo
 
 
 def e3_test_arm_stall(tile: int, wait_ns: int) -> None:
-    """Test hook: the next row call leaves one 4 KiB tile uncopied (below -1: block ``-2 - tile`` of a short call hands nothing over) and bounds
+    """Test hook: the next row call leaves one 4 KiB tile uncopied (below -1: row ``-2 - tile`` of a short call waits for a part that never comes) and bounds
     its waits by ``wait_ns``; -1 disarms it."""
     lib().e3_test_arm_stall(int(tile), int(wait_ns))
 

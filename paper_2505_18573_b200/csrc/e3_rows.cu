@@ -1188,7 +1188,7 @@ cudaError_t launch_rows(const RowsParams &p, int64_t rows, int dtype, int sample
   if (stall < 0) {  // (else the hook stalls a tile of the streaming kernel)
     if (stall < -1) stall = g_stall_tile.exchange(-1);
     bool taken = false;
-    const cudaError_t e = launch_rows_direct(p, rows, dtype, sampler, BlockStall{-2 - stall, g_stall_wait_ns.load()}, stream, taken);
+    const cudaError_t e = launch_rows_direct(p, rows, dtype, sampler, RowStall{-2 - stall, g_stall_wait_ns.load()}, stream, taken);
     if (taken || e != cudaSuccess) return e;
   }
   if (dtype == 0) {

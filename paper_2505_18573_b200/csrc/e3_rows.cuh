@@ -47,15 +47,15 @@ struct RowsParams {
   unsigned char *ws_pieces;      // [grid][2] partial states of cut rows, kPieceBytes each, every word tagged with the call id
   unsigned long long call_id;    // unique per call within the process (48 bits)
   unsigned long long wait_ns;    // time after which a wait inside the kernel gives up
-  const char *stall_src;         // test hook: the copy of the tile that begins here is never issued (short calls: the part of a row that
-                                 // begins here is not handed over); nullptr = none
+  const char *stall_src;         // test hook: the copy of the tile that begins here is never issued (short calls: the row that begins here
+                                 // waits for more than is handed over); nullptr = none
 };
 
 size_t rows_workspace_bytes();                                      // cut rows
 size_t sample_workspace_bytes(int dtype, int64_t rows, int64_t V);  // e3_sample: what the call's contract asks for
 
 // Test hook: the next launch_rows of this process gives up waiting after wait_ns and never issues the copy of
-// tile stall_tile; below -1: if it is a short call, block -2 - stall_tile never hands its part of a row over.  One shot.
+// tile stall_tile; below -1: if it is a short call, row -2 - stall_tile waits for a hand-over that never comes.  One shot.
 void arm_stall(int64_t stall_tile, unsigned long long wait_ns);
 
 // Launches the row kernel over `rows` rows (any number: more than one launch takes at a time are split).
@@ -67,10 +67,10 @@ cudaError_t launch_rows(const RowsParams &p, int64_t rows, int dtype, int sample
 // The kernel of short calls; taken: whether the call is one (if not, nothing has been launched).
 // Blocks per row that it gives such a call on a device of that many SMs whose largest cluster has `largest` blocks (0: not a short call).
 int direct_ctas(int64_t rows, int64_t V, int dtype, int sampler, bool mask, int sms, int largest);
-struct BlockStall {  // test hook: the block that hands nothing over (row * blocks per row + block; < 0: none), and the limit of the wait for it
-  long long block;
+struct RowStall {  // test hook: the row whose first block waits for more than the others hand over (< 0: none), and the limit of that wait
+  long long row;
   unsigned long long wait_ns;
 };
-cudaError_t launch_rows_direct(const RowsParams &p, int64_t rows, int dtype, int sampler, const BlockStall &stall, cudaStream_t stream, bool &taken);
+cudaError_t launch_rows_direct(const RowsParams &p, int64_t rows, int dtype, int sampler, const RowStall &stall, cudaStream_t stream, bool &taken);
 
 }  // namespace e3

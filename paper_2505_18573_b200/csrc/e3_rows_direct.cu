@@ -135,7 +135,8 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) rows_direct_kernel(
     if (rank == 0 && tid == 0) {
       mbar_init(&sh.handed, 1);
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-      mbar_arrive_expect(&sh.handed, (uint32_t)(ctas * sizeof(Part)));
+      // (test hook: 16 bytes that nobody sends)
+      mbar_arrive_expect(&sh.handed, (uint32_t)(ctas * sizeof(Part)) + (row_ptr(p, row) == p.stall_src ? 16u : 0u));
     }
     __syncwarp();
     cluster_arrive();
@@ -476,7 +477,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) rows_direct_kernel(
   }
   if (SAMPLER == 0 && pc.tb[0] >= 0) pc.zf = lds_elem<DT>(base + a + (uint32_t)((pc.tb[0] - e0) * F::kEsize));
   if (ctas > 1) {
-    if (lane < 4 && row_ptr(p, row) + (size_t)e0 * F::kEsize != p.stall_src) {
+    if (lane < 4) {
       const float x0 = lane == 0 ? pc.M : (lane == 1 ? pc.ty[0] : (lane == 2 ? __int_as_float(pc.tb[0]) : pc.zf));
       const float x1 = lane == 0 ? pc.Z : (lane == 1 ? pc.ty[1] : (lane == 2 ? __int_as_float(pc.tb[1]) : 0.f));
       const float x2 = lane == 0 ? pc.W : (lane == 1 ? pc.ty[2] : (lane == 2 ? __int_as_float(pc.tb[2]) : 0.f));
@@ -562,7 +563,7 @@ int largest_cluster(K kern, int threads) {
 }
 
 template <int DT, int SAMPLER, int kThreads>
-cudaError_t launch(const RowsParams &p, int64_t rows, int ctas, int dev, const BlockStall &stall, cudaStream_t stream, bool &taken) {
+cudaError_t launch(const RowsParams &p, int64_t rows, int ctas, int dev, const RowStall &stall, cudaStream_t stream, bool &taken) {
   static std::mutex lock;
   static int most[64];  // CTAs of a cluster; 0: not asked yet
   auto kern = rows_direct_kernel<DT, SAMPLER, kThreads>;
@@ -581,9 +582,9 @@ cudaError_t launch(const RowsParams &p, int64_t rows, int ctas, int dev, const B
   const int chunk = (int)chunk_of(p.V, ctas);
   q.wait_ns = kDefaultWaitNs;
   q.stall_src = nullptr;
-  if (stall.block >= 0) {
+  if (stall.row >= 0) {
     q.wait_ns = stall.wait_ns;
-    q.stall_src = p.logits + stall.block / ctas * p.row_bytes + stall.block % ctas * chunk * Fmt<DT>::kEsize;
+    q.stall_src = p.logits + stall.row * p.row_bytes;
   }
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -664,7 +665,7 @@ int direct_ctas(int64_t rows, int64_t V, int dtype, int sampler, bool mask, int 
   return w.ctas <= largest ? w.ctas : 0;
 }
 
-cudaError_t launch_rows_direct(const RowsParams &p, int64_t rows, int dtype, int sampler, const BlockStall &stall, cudaStream_t stream, bool &taken) {
+cudaError_t launch_rows_direct(const RowsParams &p, int64_t rows, int dtype, int sampler, const RowStall &stall, cudaStream_t stream, bool &taken) {
   static std::atomic<int> sms[64];
   taken = false;
   int dev = 0;

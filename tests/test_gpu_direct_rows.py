@@ -179,13 +179,11 @@ def test_temperatures_that_cannot_be_used_between_others(e3, dtype):
         assert_close("train.ent", en.cpu().numpy(), ren, ATOL[dtype])
 
 
-@pytest.mark.parametrize("rows, V, block", [(6, 151936, 2 * 8 + 3), (6, 151936, 5 * 8), (1, 151936, 15), (100, 20001, 99 * 2 + 1)])
+@pytest.mark.parametrize("rows, V, row", [(6, 151936, 2), (6, 151936, 5), (1, 151936, 0), (100, 20001, 99)])  # 8, 16 and 2 parts a row
 @pytest.mark.parametrize("sampler", [None, 0, 1])
-def test_a_part_that_is_never_handed_over(e3, sampler, rows, V, block):
+def test_a_part_that_is_never_handed_over(e3, sampler, rows, V, row):
     """The wait for it runs out: the row reads NaN, the status word says so, the other rows and the next call are as ever."""
-    ctas = short(e3, rows, V, torch.bfloat16, -1 if sampler is None else sampler)
-    assert ctas > 1
-    row = block // ctas
+    assert short(e3, rows, V, torch.bfloat16, -1 if sampler is None else sampler) > 1
     logits = inputs.zipf_gaussian_logits(rows, V, seed=5, dtype=torch.bfloat16, device=DEV)
     temps, targets = inputs.uniform_temps(rows, seed=6, device=DEV), inputs.uniform_targets(rows, V, seed=7, device=DEV)
     status = torch.zeros(1, dtype=torch.int32, device=DEV)
@@ -196,7 +194,7 @@ def test_a_part_that_is_never_handed_over(e3, sampler, rows, V, block):
         return e3.e3_sample(logits, temps, 3, 4, 0, sampler, status=status)
     want = run()
     assert int(status[0]) == 0
-    e3.e3_test_arm_stall(-2 - block, 5_000_000)  # 5 ms instead of two seconds
+    e3.e3_test_arm_stall(-2 - row, 5_000_000)  # 5 ms instead of two seconds
     got = run()
     assert int(status[0]) == e3.E3_STATUS_TIMEOUT
     others = torch.arange(rows, device=DEV) != row

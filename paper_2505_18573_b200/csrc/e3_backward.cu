@@ -8,7 +8,7 @@
 //
 // Work items are (row, segment), one CTA each, each thread moving 16-byte vectors (8 bf16 or 4 fp32 logits) with streaming loads and
 // stores: eight vectors per thread (32 KB of logits per item) where there are many items, because a CTA must have enough under way (bf16
-// with four: 2,048 x 151,936, 1,774 rows unmasked, 182 us, with eight 173), four where items are what there is too few of (128 x 45,000
+// with four: 2,048 x 151,936, 1,774 rows unmasked, 182 us, with eight 173 on one GPU, 199 and 188 on another), four where items are what there is too few of (128 x 45,000
 // bf16: 5.5 and 7.0 us).  What a CTA waits for before its logits is the mask alone: the row's other numbers are under way beside it, and
 // the target's logit, which needs one of them, beside the logits.  One after the other these loads cost 188 us instead of 182 on the
 // first case and 12.0 instead of 10.6 on 128 x 64,000 fp32.

@@ -62,7 +62,8 @@
 // finisher settles near-ties of block scores in fp64 and draws inside the winning block by inverse CDF (fp32, fp64 near a prefix
 // boundary).  With the scores of all blocks in a ring of shared memory instead (512 tiles of them, the variates of a segment made by the warp
 // that took its first strip, added up by atomics, looked through by the segment's finisher) strips could be four tiles long at most in
-// a long run: 4,096 x 151,936 bf16 235 us, now 216, 512 rows 41.2, now 38.3, 256 x 256,000 fp32 64.7, now 49.7.
+// a long run: 4,096 x 151,936 bf16 240-252 us, now 223-238 (two GPUs), 512 rows 41.3, now
+// 38.4, 256 x 256,000 fp32 64.5, now 49.9.
 #include "e3_rows.cuh"
 #include "e3_rows_device.cuh"
 #include "e3_rows_split.cuh"
@@ -806,8 +807,8 @@ __global__ void __launch_bounds__(kThreads, 1) rows_kernel(const __grid_constant
             float Z, W;
             float Zg[kG];
             bool summed = false;
-            // Out of line: what only few tiles need (see tile_slow).  The blocked sampler, whose short strips meet more of them, keeps
-            // all but the clamped sums in the loop.
+            // Out of line: what only few tiles need (see tile_slow).  The blocked sampler keeps all but the clamped sums in the loop (us
+            // with the careful form out of line and in the loop: 4,096 x 151,936 bf16 250, 230, 512 rows 40.1, 39.9).
             constexpr bool kLean = SAMPLER != 1;
             bool over = false;  // kLean: an entry far above the reference, or no reference yet
             if (n == F::kTileE && !(mode & kClamped)) {

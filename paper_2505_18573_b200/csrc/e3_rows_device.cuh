@@ -535,8 +535,8 @@ __device__ __forceinline__ bool careful_tile(uint32_t B, int n, float c, float &
 // entry is that low.
 // Out of line: the streaming loop stays short (bound by issue and instruction fetch).  us with it inside the loop, with the clamped
 // sums alone out of line, and with all of it: statistics 4,096 x 151,936 bf16 211, 208, 204, token sampler 512 rows 88.5, 88.5,
-// 85.5, 8 rows 28.4, 28.9, 27.0, blocked sampler 4,096 rows 252, 247, 262.  A tenth of the logits -inf, 2,048 rows, one
-// vector at a time before and now: statistics 222 and 125, blocked 248 and 161, token sampler 421 and 317.
+// 85.5; the blocked sampler 4,096 rows 230 with the clamped sums alone, 250 with all of it.  A tenth of the logits -inf, 2,048 rows, one
+// vector at a time and now: statistics 222 and 126, blocked 248 and 145, token sampler 421 and 298.
 template <int DT>
 struct SlowTile {
   float Zs, Ws, nRc;  // the strip's sums and reference, moved
